@@ -132,22 +132,22 @@ def _peaks():
 # ---------------------------------------------------------------------------
 # reference arm: the CPU oracle as it stands
 # ---------------------------------------------------------------------------
-# DRAM bytes (read + write) of the qr_chase_kernel launches of one call on
-# this workload (the chase runs in rounds, four launches per call here),
-# summed from one ncu capture of dram__bytes_read.sum + dram__bytes_write.sum;
-# valid only for the chase kernel's source it was taken with: SHA-256 of
-# qr.cu up to the first kernel after the chase (the deferred-pass kernels and
-# the host code follow it) plus common.cuh, else null.
-CHASE_TRAFFIC = {"sha256": "d1f1d12129d4a9b51dcd2a46ba065b813269b030c5a66f7354d23ac5d53f33f0", "bytes": 4572416}
-_CHASE_END = "__global__ void __launch_bounds__(128) qr_build_u_kernel"
+# DRAM bytes (read + write) of the rqr_chase_kernel launches of one call on
+# this workload (the chase runs in rounds, one launch each), summed from one
+# ncu capture of dram__bytes_read.sum + dram__bytes_write.sum; valid only for
+# the chase kernel's source it was taken with: SHA-256 of rqr.cu up to the
+# first kernel after the chase (the deferred-pass kernels and the host code
+# follow it) plus qr_small.cuh and common.cuh, else null.
+CHASE_TRAFFIC = {"sha256": "e17cbf10c3ff25fd059eaa3729eb6fccaaf7f9fd41ad1a9d4c39bc71c7248891", "bytes": 1637120}
+_CHASE_END = "__global__ void __launch_bounds__(kBuildThreads) rqr_build_u_kernel"
 
 
 def _chase_traffic():
     import hashlib
     d = os.path.join(os.path.dirname(os.path.abspath(__file__)), "paper_2607_12430_gb300", "csrc")
     try:
-        q = open(os.path.join(d, "qr.cu")).read()
-        c = open(os.path.join(d, "common.cuh")).read()
+        q = open(os.path.join(d, "rqr.cu")).read()
+        c = open(os.path.join(d, "qr_small.cuh")).read() + open(os.path.join(d, "common.cuh")).read()
     except OSError:
         return None
     if _CHASE_END not in q:
@@ -355,7 +355,7 @@ def leg_set_iii(args, mp, torch, flush, fp32_peak_tflops):
     ts, (_, info) = _timed_calls(torch, lambda: mp.sqrtm_mixed(A, kind=mp.KIND_GENERAL, steps=kstar, out=X),
                                  reps, flush)
     ms = statistics.mean(ts)
-    chase_flops = 20.0 * info["schur_work"]
+    chase_flops = 10.0 * info["schur_work"]
     achieved = chase_flops / (info["ms_qr_chase"] * 1e-3) / 1e12
     return {"workload": "Table 1 set III: U(0,1) n=4096 plus shift (real eigenvalues >= 1), seed 20260712+10",
             "n": n, "target": 1e-12, "k_star": kstar, "forward_error": errs[kstar], "errors_by_step": errs,
@@ -366,7 +366,7 @@ def leg_set_iii(args, mp, torch, flush, fp32_peak_tflops):
                           "ms_qr_chase": info["ms_qr_chase"], "ms_trisqrt": info["ms_trisqrt"],
                           "ms_refine": info["ms_refine"]},
             "schur_sweeps": info["schur_sweeps"], "schur_rotations": info["schur_rotations"],
-            "roofline": {"kernel": "qr_chase_kernel<float>", "bound": "alu", "achieved": achieved,
+            "roofline": {"kernel": "rqr_chase_kernel<1>", "bound": "alu", "achieved": achieved,
                          "peak": fp32_peak_tflops, "unit": "TFLOP/s", "frac": achieved / fp32_peak_tflops,
                          "traffic": None, "flops_per_call": chase_flops},
             "input_prep_s": gen_s}
@@ -498,32 +498,31 @@ def run_ours(args):
 
     # ---- roofline of the dominant kernel: the QR chase ----
     peaks = _peaks()
-    # Algorithmic work, counted by the kernel: every rotation of a sweep on the
-    # active block [lo, hi] rotates about m = hi - lo + 1 pairs of complex
-    # entries of T (two rows right of it, two columns above it); a complex
-    # rotation of one pair, (c p + s q, c q - conj(s) p) with c real, costs 20
-    # real flops.  The duration is the sum of the chase kernel's launches,
+    # Algorithmic work, counted by the kernel: every reflector of a sweep on the
+    # active block [lo, hi] updates about m = hi - lo + 1 segments of three
+    # entries of the real T (three rows right of it, three columns above it); a
+    # segment, x - tau (v^T x) v with v = (1, v1, v2), costs 10 flops.  The duration is the sum of the chase kernel's launches,
     # timed with CUDA events on the library's stream inside the timed steps.
     work = statistics.mean([i["schur_work"] for i in infos])
     chase_ms = statistics.mean([i["ms_qr_chase"] for i in infos])
-    chase_flops = 20.0 * work
+    chase_flops = 10.0 * work
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
     mhz = clocks.get("sm_max_mhz") or peaks.get("sm_max_mhz") or 2070.0
     # FP32 FFMA lanes (128 per SM on sm_103) x 2 flops x the device's maximum SM clock
     fp32_peak_tflops = sms * 128 * 2 * mhz * 1e6 / 1e12
     one_sm_peak = fp32_peak_tflops / sms
     achieved = chase_flops / (chase_ms * 1e-3) / 1e12
-    roofline = {"kernel": "qr_chase_kernel<float>", "bound": "alu", "achieved": achieved,
+    roofline = {"kernel": "rqr_chase_kernel<1>", "bound": "alu", "achieved": achieved,
                 "peak": fp32_peak_tflops, "unit": "TFLOP/s", "frac": achieved / fp32_peak_tflops,
                 "traffic": _chase_traffic(),
                 "kernel_ms_per_step": chase_ms, "flops_per_step": chase_flops,
                 "peak_one_sm": one_sm_peak, "frac_one_sm": achieved / one_sm_peak,
                 "note": f"peak derived ({sms} SMs x 128 FP32 lanes x 2 flop x {mhz:.0f} MHz, read from the "
                         "device), not measured; the "
-                        "bulge chain runs on one chase CTA (8 helper CTAs take the out-of-window "
+                        "bulge chain runs on one chase CTA (16 helper CTAs take the out-of-window "
                         "updates), so the one-SM fraction is the meaningful one; achieved and traffic "
                         "are per step, summed over the chase launches of one call (ncu dram bytes, "
-                        "for this qr.cu only)"}
+                        "for this rqr.cu only)"}
 
     line = {
         "metric": METRIC, "value": ms, "unit": "ms", "n_gpus": ws, "steps": args.steps,

@@ -127,12 +127,15 @@ typedef struct {
     double ms_schur, ms_trisqrt, ms_refine;
     /* of ms_schur: the Hessenberg (or tridiagonal) reduction alone */
     double ms_reduction;
-    /* QR sweeps and Givens rotations of the Schur iteration (general path) */
+    /* QR sweeps and rotations of the Schur iteration (general path; a real
+     * matrix in FP32: 3 x 3 reflectors, one per two shifts, and the rotations
+     * of its small diagonal blocks) */
     int schur_sweeps;
     int64_t schur_rotations;
     /* general path: summed duration of the QR chase kernel's launches (ms)
      * and its in-block work, sum over sweeps of rotations x active-block
-     * size (each such unit is one rotated pair of complex entries) */
+     * size (each such unit is one rotated pair of complex entries; a real
+     * matrix in FP32: one segment of three entries, reflected) */
     double ms_qr_chase;
     int64_t schur_work;
 } sqrtm_info;

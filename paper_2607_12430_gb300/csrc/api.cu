@@ -359,7 +359,7 @@ static int general_path(sqrtm_handle_t h, const double *dA, int64_t n, int64_t l
                     Carve::round(2 * sizeof(SchurDesc<R>)) +
                     2 * (Carve::round(qr_log_capacity(n) * sizeof(RotLog<R>)) +
                          Carve::round(qr_win_capacity(n) * sizeof(WinRec)) + Carve::round(qr_u_capacity(n) * cb)) +
-                    Carve::round(kQrStateInts * sizeof(int)) + Carve::round(4 * sizeof(int)) + Carve::round(32 * sizeof(int)) + Carve::round(qr_win_capacity(n) * sizeof(int)) + 4096 +
+                    Carve::round(kQrStateInts * sizeof(int)) + Carve::round(4 * sizeof(int)) + Carve::round(kQrSyncInts * sizeof(int)) + Carve::round(qr_win_capacity(n) * sizeof(int)) + 4096 +
                     (root == 3 ? Carve::round(nn * cb) : 0) + Carve::round(rtrsyl_flow_ints((int)n, (int)n) * sizeof(int));
     // split-TF32 tensor-core transforms (X_0 = Q S Q^H, R~ = Q^H Rhat Q,
     // X += Re(Q Y Q^H)) for the FP32 square root of a real matrix of even
@@ -408,7 +408,7 @@ static int general_path(sqrtm_handle_t h, const double *dA, int64_t n, int64_t l
     }
     int *qstate = cw.take<int>(kQrStateInts);
     int *rstate = cw.take<int>(4);
-    int *qsync = cw.take<int>(32);
+    int *qsync = cw.take<int>(kQrSyncInts);
     int *qpost = cw.take<int>(qr_win_capacity(n));
     // cube root: V = S^2 beside S; X X in FP64 shares Rt's bytes (it is read
     // by the residual before Rt is next written)
@@ -450,7 +450,7 @@ static int general_path(sqrtm_handle_t h, const double *dA, int64_t n, int64_t l
     if (norm_a == 0.0) return 2;  // the zero matrix has the eigenvalue 0
 
     SchurDesc<R> hd;
-    hd.T = T; hd.Q = Q; hd.v = v; hd.beta = beta; hd.status = sc.st_schur; hd.n = (int)n; hd.ld = (int)n;
+    hd.T = T; hd.Q = Q; hd.v = v; hd.beta = beta; hd.w = W; hd.status = sc.st_schur; hd.n = (int)n; hd.ld = (int)n;
     hd.counters = sc.st_schur + 3;
     hd.state = qstate; hd.log_cap = (int)std::min<int64_t>(qr_log_capacity(n), INT32_MAX);
     // rounds of at most max(64, n/2) windows, so that several rounds overlap
@@ -500,8 +500,18 @@ static int general_path(sqrtm_handle_t h, const double *dA, int64_t n, int64_t l
     SQM_CU(cudaEventRecord(ev_red, s));
     float ms_chase = 0.0f;
     const sqrtm_tune_entry *tune = tune_for(h, n);
-    SQM_CU(launch_qr_sweeps<R>(ddesc, 1, (int)n, (int *)h->staging.p + 512, qstate, s, &ms_chase, ddesc + 1, h->side,
-                               h->qev, qsync, tune ? tune->qr_helpers : -1));
+    // A real and FP32: the iteration runs in real arithmetic (W is free)
+    bool real_qr = false;
+    if constexpr (sizeof(R) == sizeof(float)) {
+        if (!cin) {
+            real_qr = true;
+            SQM_CU(launch_rqr_sweeps(ddesc, (int)n, (int *)h->staging.p + 512, qstate, s, &ms_chase, ddesc + 1, h->side,
+                                     h->qev, qsync, tune ? tune->qr_helpers : -1));
+        }
+    }
+    if (!real_qr)
+        SQM_CU(launch_qr_sweeps<R>(ddesc, 1, (int)n, (int *)h->staging.p + 512, qstate, s, &ms_chase, ddesc + 1, h->side,
+                                   h->qev, qsync, tune ? tune->qr_helpers : -1));
     SQM_CU(cudaEventRecord(h->ev[1], s));
     if (root == 3) SQM_CU(launch_tricbrt<R>(T, (int)n, S, (int)n, V, (int)n, (int)n, o.blks, sc.st_solve, s));
     else if (tune && tune->trisqrt_cutoff > 0 && n > tune->trisqrt_cutoff)

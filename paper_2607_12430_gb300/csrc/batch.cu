@@ -518,7 +518,8 @@ cudaError_t enqueue_pipeline(void *p, cudaStream_t s)
         i0 = i1;
     }
     bstamp_kernel<<<1, 1, 0, s>>>(L.stamps, 1); count_launch();
-    if (Bg > 0 && (err = enqueue_qr_sweeps_device<R>(L.desc, Bg, c->nord[0], &L.prm->round, s, c->body_stream)))
+    if (Bg > 0 && (err = enqueue_rqr_sweeps_device(L.desc, Bg, c->nord[0], c->nord[Bg - 1], &L.prm->round, s,
+                                                     c->body_stream)))
         return err;
     bstamp_kernel<<<1, 1, 0, s>>>(L.stamps, 2); count_launch();
     // symmetric members: Jacobi, V in global memory above kJacVsmemMaxN
@@ -679,7 +680,7 @@ int batched_general(sqrtm_handle_t h, const int *idx, int count, const double *c
         d.state = L.qstate + kQrStateInts * (size_t)i;
         d.log_cap = (int)std::min<int64_t>(qr_log_capacity(nm), INT32_MAX);
         d.win_cap = (int)std::min<int64_t>(qr_win_capacity(nm), INT32_MAX);
-        d.T = T; d.Q = Q; d.n = (int)nm; d.ld = (int)nm;
+        d.T = T; d.Q = Q; d.w = W; d.n = (int)nm; d.ld = (int)nm;
         BState *q = L.st + i;
         d.status = &q->st_schur;
         htri[i] = TriJob<R>{T, S, Rt, &q->st_solve, &q->active, (int)nm};

@@ -63,6 +63,7 @@ struct SchurDesc {
     cplx<R> *Q;      // out: unitary Schur vectors (n x n)
     cplx<R> *v;      // scratch: Householder vector (>= n entries)
     R *beta;         // scratch: reflector scalars [beta, |x|, phase.x, phase.y]
+    cplx<R> *w = nullptr;  // scratch (real QR iteration): n x n complex, the real H then T and Q
     int *status;     // out: 0 / 3 (iteration cap)
     int *counters;   // out (7 ints): [0] sweeps, [1..2] rotations, [3..4] the chase kernel's in-block
                      // rotation work (int64s split lo/hi); cooperative chase: [5] sweeps and [6]
@@ -175,17 +176,25 @@ cudaError_t launch_hessenberg_cluster_batched(const HessJob<R> *jobs, int count,
 // sets and each round's deferred passes run on `side` (ordered by the four
 // events qev) while the next round's chase runs on s.  The deferred passes
 // touch only T entries outside every later active block and Z, which the
-// chase never reads.  d_sync (may be null; >= 32 ints, the descriptors'
+// chase never reads.  d_sync (may be null; kQrSyncInts, the descriptors'
 // `sync`): with batch == 1 and a large enough n the chase runs as one
 // cooperative grid of a chase CTA and helper CTAs that take the
 // out-of-window updates of the active block.  helpers: number of helper
 // CTAs (0: no cooperative grid; -1: 8, 16 from n = 1024).
 constexpr int kQrStateInts = 16;
+constexpr int kQrSyncInts = 96;  // counters of a cooperative chase (d_sync)
 template <class R>
 cudaError_t launch_qr_sweeps(const SchurDesc<R> *d_desc, int batch, int nmax, int *h_state,
                              const int *d_state_all, cudaStream_t s, float *ms_chase = nullptr,
                              const SchurDesc<R> *d_desc_alt = nullptr, cudaStream_t side = nullptr,
                              const cudaEvent_t *qev = nullptr, int *d_sync = nullptr, int helpers = -1);
+// The same for a REAL matrix in FP32 (rqr.cu): T and Q hold the Hessenberg
+// form and its Q with zero imaginary parts and receive the complex Schur
+// form; the iteration itself runs in real arithmetic on copies in the
+// descriptors' w, and v holds the block starts.  d_state: one state block.
+cudaError_t launch_rqr_sweeps(const SchurDesc<float> *d_desc, int n, int *h_state, const int *d_state, cudaStream_t s,
+                              float *ms_chase, const SchurDesc<float> *d_desc_alt, cudaStream_t side,
+                              const cudaEvent_t *qev, int *d_sync, int helpers);
 // Real Householder Hessenberg reduction of a real matrix of any size
 // (schur.cu): from the real parts of the complex A_s in T, H (real, ld n)
 // becomes upper Hessenberg and Qr = P_0 ... P_{n-3} (real, ld n); Y
@@ -209,14 +218,13 @@ cudaError_t launch_hessenberg_real_finish(const R *H, const R *Qr, cplx<R> *T, c
 typedef cudaError_t (*CondFn)(void *ctx, cudaStream_t st, cudaGraphConditionalHandle cond);
 cudaError_t capture_while(cudaStream_t s, cudaStream_t body_stream, unsigned init, CondFn body, void *ctx,
                           CondFn pre = nullptr);
-// The QR rounds of a batch for capture into a graph: state initialisation,
-// a WHILE node whose body is one round (chase with one CTA per matrix,
-// window products, deferred passes, and a one-thread test of every
-// matrix's done flag; at most 256 rounds, then status 3), and the final
-// clean-up of T.  d_round: one device int of scratch.
-template <class R>
-cudaError_t enqueue_qr_sweeps_device(const SchurDesc<R> *d_desc, int batch, int nmax, int *d_round, cudaStream_t s,
-                                     cudaStream_t body_stream);
+// The real QR rounds of a batch (sizes nmin .. nmax) for capture into a
+// graph: real copies and state, a WHILE node whose body is one round (chase
+// with one CTA per matrix, window products, deferred passes, and a test of
+// every matrix's done flag; at most 256 rounds, then status 3), and the
+// complex Schur form of the diagonal blocks.  d_round: one device int.
+cudaError_t enqueue_rqr_sweeps_device(const SchurDesc<float> *d_desc, int batch, int nmax, int nmin, int *d_round,
+                                      cudaStream_t s, cudaStream_t body_stream);
 // scratch sizes per matrix of size n: rotation log entries, window records,
 // elements of accumulated window products (one round of the QR iteration
 // stops at a sweep boundary before any of them would overflow)
