@@ -267,10 +267,182 @@ __global__ void tri_finish_kernel(R *__restrict__ A, int n, int ld, const R *__r
     }
 }
 
+// The same reduction of a matrix that fits one CTA's shared memory, in one
+// launch: warp 0 forms w, updates column k + 1 and makes its reflector (the
+// vectors of at most 32 TRI_RPL entries in registers, shuffles for the sums),
+// then every warp applies the rank-2 update to its columns and takes their
+// products with the new reflector.  Two barriers per column in place of a
+// launch: bound by warp 0's serial part (two sums over the warp, a square root
+// and a division) and, for larger n, by the shared-memory pass over the block;
+// FP64 by the FP64 units of the one SM.  One CTA because a column's work is
+// less than what a second CTA's exchange would cost; an odd leading dimension
+// so that columns start in different banks.  Measured: see launch_tridiag.
+static constexpr int kTriSmallThreads = 1024;
+template <class R> struct TriSmall;
+template <> struct TriSmall<float> { static constexpr int maxn = 224; };
+template <> struct TriSmall<double> { static constexpr int maxn = 96; };
+
+template <class R>
+__host__ __device__ __forceinline__ int tri_small_ld(int n) { return n | 1; }
+
+template <class R>
+__global__ void __launch_bounds__(kTriSmallThreads, 1)
+tri_small_kernel(R *__restrict__ A, int n, int ld, R *__restrict__ Y, int ldy, R *__restrict__ betas)
+{
+    constexpr int RPL = (TriSmall<R>::maxn + 31) / 32;
+    extern __shared__ unsigned char smraw[];
+    const int lds = tri_small_ld<R>(n);
+    R *S = reinterpret_cast<R *>(smraw);  // S[i + j lds]
+    R *v = S + (size_t)lds * n, *w = v + n, *p = w + n, *vn = p + n;
+    __shared__ R s_bn;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    constexpr int NW = kTriSmallThreads / 32;
+    for (int j = warp; j < n; j += NW)
+        for (int i = lane; i < n; i += 32) S[i + j * lds] = A[i + (int64_t)j * ld];
+    for (int i = tid; i < n; i += kTriSmallThreads) v[i] = w[i] = p[i] = R(0);
+    __syncthreads();
+    R beta = 0;  // of the step before (warp 0)
+    // step k: the rank-2 update of reflector k - 1 on rows and columns >= k
+    // (v, p = beta S v of that reflector; none for k = 0) and reflector k
+    for (int k = 0; k + 1 < n; ++k) {
+        if (warp == 0) {
+            R vr[RPL], pr[RPL], c[RPL];
+            R acc = 0;
+#pragma unroll
+            for (int q = 0; q < RPL; ++q) {
+                const int i = lane + 32 * q;
+                const bool in = i >= k && i < n;
+                vr[q] = in ? v[i] : R(0);
+                pr[q] = in && beta != R(0) ? p[i] : R(0);
+                c[q] = in ? S[i + k * lds] : R(0);
+                acc = fma(vr[q], pr[q], acc);
+            }
+            acc = warp_sum(acc);
+            const R K = R(0.5) * beta * acc;
+            R v0 = 0, w0 = 0;
+#pragma unroll
+            for (int q = 0; q < RPL; ++q) {
+                pr[q] = fma(-K, vr[q], pr[q]);  // w
+                const int i = lane + 32 * q;
+                if (i >= k && i < n) w[i] = pr[q];
+                if (q == (k >> 5)) { v0 = vr[q]; w0 = pr[q]; }
+            }
+            v0 = __shfl_sync(0xffffffffu, v0, k & 31);
+            w0 = __shfl_sync(0xffffffffu, w0, k & 31);
+            // column k and its reflector
+            R tail = 0, x0 = 0;
+#pragma unroll
+            for (int q = 0; q < RPL; ++q) {
+                const int i = lane + 32 * q;
+                c[q] = fma(-vr[q], w0, fma(-pr[q], v0, c[q]));
+                if (i == k) S[k + k * lds] = c[q];  // final diagonal entry
+                if (i > k + 1 && i < n) tail = fma(c[q], c[q], tail);
+                if (q == ((k + 1) >> 5)) x0 = c[q];
+            }
+            tail = warp_sum(tail);
+            x0 = __shfl_sync(0xffffffffu, x0, (k + 1) & 31);
+            R bn = 0, sub = x0, y0 = 0;
+            if (tail != R(0) && k + 2 < n) {
+                const R xn = sqrt(fma(x0, x0, tail)), sg = x0 >= R(0) ? R(1) : R(-1);
+                y0 = x0 + sg * xn;
+                bn = R(2) / (y0 * y0 + tail);
+                sub = -sg * xn;
+            }
+#pragma unroll
+            for (int q = 0; q < RPL; ++q) {
+                const int i = lane + 32 * q;
+                if (i > k && i < n) {
+                    const R y = i == k + 1 ? y0 : (k + 2 < n ? c[q] : R(0));
+                    vn[i] = y;
+                    if (k + 2 < n) Y[i + (int64_t)k * ldy] = y;
+                }
+            }
+            if (lane == 0) {
+                S[(k + 1) + k * lds] = sub;
+                if (k + 2 < n) betas[k] = bn;
+                s_bn = bn;
+            }
+            beta = bn;
+        }
+        __syncthreads();
+        const R bn = s_bn;
+        // columns > k, two at a time in FP32 (latency) and one in FP64 (whose
+        // units a second, idle column would still occupy): rank-2 update and
+        // product with the new reflector, the three vectors in registers over
+        // the columns (a row at or above k meets zeros in all three)
+        constexpr int C = sizeof(R) == 4 ? 2 : 1;
+        R vr[RPL], wr[RPL], yr[RPL];
+#pragma unroll
+        for (int q = 0; q < RPL; ++q) {
+            const int i = lane + 32 * q;
+            const bool in = i > k && i < n;
+            vr[q] = in ? v[i] : R(0);
+            wr[q] = in ? w[i] : R(0);
+            yr[q] = in ? vn[i] : R(0);
+        }
+        const int q0 = (k + 1) >> 5;
+#pragma unroll 1
+        for (int j = k + 1 + warp; j < n; j += C * NW) {
+            int jc[C];
+            R vj[C], wj[C], dot[C];
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                jc[c] = j + c * NW < n ? j + c * NW : j;
+                vj[c] = v[jc[c]];
+                wj[c] = w[jc[c]];
+                dot[c] = 0;
+            }
+#pragma unroll
+            for (int q = 0; q < RPL; ++q) {
+                const int i = lane + 32 * q;
+                if (q < q0 || i >= n) continue;
+                R x[C];
+#pragma unroll
+                for (int c = 0; c < C; ++c) {
+                    x[c] = fma(-vr[q], wj[c], fma(-wr[q], vj[c], S[i + jc[c] * lds]));
+                    dot[c] = fma(x[c], yr[q], dot[c]);
+                }
+#pragma unroll
+                for (int c = 0; c < C; ++c) S[i + jc[c] * lds] = x[c];  // the same value twice where jc is j
+            }
+#pragma unroll
+            for (int o = 16; o; o >>= 1)
+#pragma unroll
+                for (int c = 0; c < C; ++c) dot[c] += __shfl_xor_sync(0xffffffffu, dot[c], o);
+            if (lane == 0) {
+#pragma unroll
+                for (int c = 0; c < C; ++c) p[jc[c]] = bn * dot[c];
+            }
+        }
+        R *t = v;
+        v = vn;
+        vn = t;
+        __syncthreads();
+    }
+    // the last diagonal entry took its updates in the passes above
+    for (int i = tid; i < n; i += kTriSmallThreads) {
+        A[i + (int64_t)i * ld] = S[i + i * lds];
+        if (i + 1 < n) A[(i + 1) + (int64_t)i * ld] = S[(i + 1) + i * lds];
+    }
+}
+
 template <class R>
 cudaError_t launch_tridiag(R *A, int n, int ld, R *Y, int ldy, R *betas, R *ws, cudaStream_t s)
 {
     if (n < 3) return cudaSuccess;
+    // In one CTA while the matrix fits its shared memory (FP32: n <= 224) and
+    // one SM's FP64 units keep up (FP64: n <= 96, where the gain has fallen to
+    // 28 %).  In one CTA against a launch per column, ms of reduction: FP32
+    // n = 64 0.156 / 0.275, 128 0.313 / 0.491, 224 0.674 / 0.853; FP64 n = 64
+    // 0.484 / 0.842, 96 0.908 / 1.254.
+    if (n <= TriSmall<R>::maxn) {
+        const size_t smem = ((size_t)tri_small_ld<R>(n) * n + 4 * (size_t)n) * sizeof(R);
+        cudaError_t e = allow_max_smem((const void *)tri_small_kernel<R>);
+        if (e) return e;
+        tri_small_kernel<R><<<1, kTriSmallThreads, smem, s>>>(A, n, ld, Y, ldy, betas);
+        count_launch();
+        return cudaGetLastError();
+    }
     // two sets of (v, p, scalars), alternating between steps
     R *set[2] = {ws, ws + 2 * n + 8};
     size_t sm1 = (size_t)n * sizeof(R);
