@@ -121,7 +121,9 @@ template <int U = 8, class LD, class ST>
 __device__ __forceinline__ void copy_cols(int rows, int cols, int warp, int nw, LD load, ST store)
 {
     const int lane = threadIdx.x & 31;
+#pragma unroll 1
     for (int b0 = warp * U; b0 < cols; b0 += nw * U)
+#pragma unroll 1
         for (int a = lane; a < rows; a += 32) {
             float v[U];
 #pragma unroll
@@ -224,7 +226,7 @@ __device__ __forceinline__ void tile_update(float a[3][3], Refl l, Refl r)
 // First reflector of a bulge with shifts alpha +- sqrt(-q): from the first
 // column of (H - s1)(H - s2) for the block starting at lo.  B(i, j) is
 // element (i, j) at B[i + j ld].
-__device__ __forceinline__ Refl intro_reflector(const float *B, int ld, int lo, float alpha, float q)
+__device__ __noinline__ Refl intro_reflector(const float *B, int ld, int lo, float alpha, float q)
 {
     const float a = B[lo + lo * ld], b = B[lo + (lo + 1) * ld], c = B[(lo + 1) + lo * ld],
                 d = B[(lo + 1) + (lo + 1) * ld], e = B[(lo + 2) + (lo + 1) * ld];
@@ -255,8 +257,11 @@ __device__ __forceinline__ int prog_get(const int *p)
 // The diagonal tiles during a window (steps t0 .. t1 - 1; element (i, j) at
 // B[i + j ld]), lane g: bulge g.  rt: the window's table, row 0 given; every
 // step writes the next one's row, the last one rt_next's row 0.  Entries
-// below the subdiagonal that a bulge has left are not cleared: nothing reads
-// them.
+// below the subdiagonal that a bulge has left are not cleared: nothing uses
+// them.  One path for every step, entering and leaving bulges included: the
+// chase kernels' code has to stay within the instruction caches (as separate
+// steady and general paths, 130 KB in all, a step took 600 cycles in the
+// kernel and the first iteration of each shift computation 40 k).
 __device__ __forceinline__ void diag_window(float *B, int ld, int lo, int hi, int t0, int t1, int nb, float *rt,
                                             float *rt_next, const float2 *s_sh)
 {
@@ -268,174 +273,103 @@ __device__ __forceinline__ void diag_window(float *B, int ld, int lo, int hi, in
         for (int c = 0; c < 3; ++c) a[q][c] = 0.0f;
     Refl v{0.0f, 0.0f, 0.0f};
     if (g < NB) v = table_get(rt, g);
-    // held: a holds columns p, p + 1 of the tile with the left reflector
-    // already applied to them (before the barrier, in the shadow of the
-    // stores), and s the sums a_q0 + v1 a_q1
-    bool held = false;
+    // a holds columns p, p + 1 of the tile with the left reflector already
+    // applied to them (before the barrier, in the shadow of the stores), s the
+    // sums a_q0 + v1 a_q1
     float s0 = 0.0f, s1 = 0.0f, s2 = 0.0f;
-    auto left2 = [&]() {
-#pragma unroll
-        for (int c = 0; c < 2; ++c) {
-            const float w = v.z * fmaf(v.y, a[2][c], fmaf(v.x, a[1][c], a[0][c]));
-            a[0][c] -= w;
-            a[1][c] = fmaf(-w, v.x, a[1][c]);
-            a[2][c] = fmaf(-w, v.y, a[2][c]);
-        }
-        s0 = fmaf(v.x, a[0][1], a[0][0]);
-        s1 = fmaf(v.x, a[1][1], a[1][0]);
-        s2 = fmaf(v.x, a[2][1], a[2][0]);
-    };
-    // column p + 2 and the right reflector; f: the subdiagonal entry below
-    auto finish = [&](float f, float &f0, float &f1, float &f2) {
-        const float w = v.z * fmaf(v.y, a[2][2], fmaf(v.x, a[1][2], a[0][2]));
-        a[1][2] = fmaf(-w, v.x, a[1][2]);
-        a[2][2] = fmaf(-w, v.y, a[2][2]);
-        a[0][2] -= w;
-        const float w1 = v.z * fmaf(v.y, a[1][2], s1), w2 = v.z * fmaf(v.y, a[2][2], s2), w0 = v.z * fmaf(v.y, a[0][2], s0);
-        a[1][0] -= w1;
-        a[2][0] -= w2;
-        a[0][0] -= w0;
-        const float u = v.z * v.y * f;
-        f0 = -u;
-        f1 = -u * v.x;
-        f2 = fmaf(-u, v.y, f);
-        a[1][1] = fmaf(-w1, v.x, a[1][1]);
-        a[2][1] = fmaf(-w2, v.x, a[2][1]);
-        a[0][1] = fmaf(-w0, v.x, a[0][1]);
-        a[1][2] = fmaf(-w1, v.y, a[1][2]);
-        a[2][2] = fmaf(-w2, v.y, a[2][2]);
-        a[0][2] = fmaf(-w0, v.y, a[0][2]);
-    };
-    auto shift = [&](float f1, float f2) {
-        a[0][0] = a[1][1];
-        a[0][1] = a[1][2];
-        a[1][0] = a[2][1];
-        a[1][1] = a[2][2];
-        a[2][0] = f1;
-        a[2][1] = f2;
-    };
-    // a step with every bulge on its way and inside the block, the tiles held;
-    // f1, f2: what the next tile's last row takes over
-    auto steady = [&](int t, float *row, float &f1, float &f2) {
-        const int p = lo + t - 3 * g;
-        float *e = B + p + p * ld;
-#pragma unroll
-        for (int q = 0; q < 3; ++q) a[q][2] = e[q + 2 * ld];
-        const float f = e[3 + 2 * ld];
-        float f0, beta;
-        finish(f, f0, f1, f2);
-        e[0] = a[0][0];
-        e[ld] = a[0][1];
-        e[2 * ld] = a[0][2];
-        Refl nxt;
-        reflector3(a[1][0], a[2][0], f0, nxt, beta);
-        table_put(row, g, nxt);
-        e[1] = beta;
-        v = nxt;
-    };
-    if (t0 > 3 * (nb - 1) && lo + t1 + 2 <= hi) {  // a whole window of such steps
-        float f1 = 0.0f, f2 = 0.0f;
-        if (g < nb) {
-            const float *e = B + (lo + t0 - 3 * g) * (1 + ld);
-#pragma unroll
-            for (int c = 0; c < 2; ++c)
-#pragma unroll
-                for (int q = 0; q < 3; ++q) a[q][c] = e[q + c * ld];
-            left2();
-        }
-        for (int t = t0; t + 1 < t1; ++t) {
-            float *row = rt + (t + 1 - t0) * TS;
-            if (g < nb) {
-                steady(t, row, f1, f2);
-                shift(f1, f2);
-                left2();
-            } else if (g < NB) {
-                table_put(row, g, v);  // (zero)
-            }
-            step_bar();
-        }
-        if (g < nb) {
-            steady(t1 - 1, rt_next, f1, f2);
-            float *e = B + (lo + t1 - 1 - 3 * g) * (1 + ld);
-            e[1 + ld] = a[1][1];
-            e[2 + ld] = a[2][1];
-            e[3 + ld] = f1;
-            e[1 + 2 * ld] = a[1][2];
-            e[2 + 2 * ld] = a[2][2];
-            e[3 + 2 * ld] = f2;
-        } else if (g < NB) {
-            table_put(rt_next, g, v);
-        }
-        step_bar();
-        return;
-    }
+    bool held = false;
+#pragma unroll 1
     for (int t = t0; t < t1; ++t) {
-        if (t > 3 * (nb - 1) && t > t0 && t + 1 < t1 && lo + t + 3 <= hi) {
-            float *row = rt + (t + 1 - t0) * TS;
-            if (g < nb) {
-                float f1, f2;
-                steady(t, row, f1, f2);
-                shift(f1, f2);
-                left2();
-            } else if (g < NB) {
-                table_put(row, g, v);
-            }
-            step_bar();
-            continue;
-        }
         if (g < NB) {
             const int p = lo + t - 3 * g;
             float *row = t + 1 < t1 ? rt + (t + 1 - t0) * TS : rt_next;
-            Refl nxt{0.0f, 0.0f, 0.0f};
-            if (g < nb && p >= lo && p < hi) {
-                float *e = B + p + p * ld;
-                const bool k2 = p + 2 <= hi, k3 = p + 3 <= hi;
-                if (!held) {
+            float *e = B + p + p * ld;
+            const bool act = g < nb && p >= lo && p < hi, k2 = act && p + 2 <= hi, k3 = act && p + 3 <= hi;
+            if (act && !held) {
 #pragma unroll
-                    for (int c = 0; c < 2; ++c)
+                for (int c = 0; c < 2; ++c)
 #pragma unroll
-                        for (int q = 0; q < 3; ++q) a[q][c] = (k2 || q < 2) ? e[q + c * ld] : 0.0f;
-                    if (p == lo) a[2][0] = 0.0f;  // (a bulge that enters: not cleared by the one before)
-                    left2();
-                    held = true;
+                    for (int q = 0; q < 3; ++q) a[q][c] = (k2 || q < 2) ? e[q + c * ld] : 0.0f;
+                if (p == lo) a[2][0] = 0.0f;  // (a bulge that enters: not cleared by the one before)
+#pragma unroll
+                for (int c = 0; c < 2; ++c) {
+                    const float w = v.z * fmaf(v.y, a[2][c], fmaf(v.x, a[1][c], a[0][c]));
+                    a[0][c] -= w;
+                    a[1][c] = fmaf(-w, v.x, a[1][c]);
+                    a[2][c] = fmaf(-w, v.y, a[2][c]);
                 }
+                s0 = fmaf(v.x, a[0][1], a[0][0]);
+                s1 = fmaf(v.x, a[1][1], a[1][0]);
+                s2 = fmaf(v.x, a[2][1], a[2][0]);
+                held = true;
+            }
+            // column p + 2 and the right reflector; f: the subdiagonal entry below
+            float f = 0.0f;
 #pragma unroll
-                for (int q = 0; q < 3; ++q) a[q][2] = k2 ? e[q + 2 * ld] : 0.0f;
-                const float f = k3 ? e[3 + 2 * ld] : 0.0f;
-                float f0, f1, f2;
-                finish(f, f0, f1, f2);
-                if (k2) {  // p + 1 <= hi - 1: column p defines the next reflector
-                    float beta;
-                    reflector3(a[1][0], a[2][0], f0, nxt, beta);
-                    a[1][0] = beta;
-                }
-                table_put(row, g, nxt);
-                // row p and column p leave the tile
+            for (int q = 0; q < 3; ++q) a[q][2] = 0.0f;
+            if (k2) {
+#pragma unroll
+                for (int q = 0; q < 3; ++q) a[q][2] = e[q + 2 * ld];
+            }
+            if (k3) f = e[3 + 2 * ld];
+            const float w = v.z * fmaf(v.y, a[2][2], fmaf(v.x, a[1][2], a[0][2]));
+            a[1][2] = fmaf(-w, v.x, a[1][2]);
+            a[2][2] = fmaf(-w, v.y, a[2][2]);
+            a[0][2] -= w;
+            const float w1 = v.z * fmaf(v.y, a[1][2], s1), w2 = v.z * fmaf(v.y, a[2][2], s2),
+                        w0 = v.z * fmaf(v.y, a[0][2], s0);
+            a[1][0] -= w1;
+            a[2][0] -= w2;
+            const float u = v.z * v.y * f;
+            // column p defines the next reflector
+            Refl nxt;
+            float beta;
+            reflector3(a[1][0], a[2][0], -u, nxt, beta);
+            a[0][0] -= w0;
+            a[0][1] = fmaf(-w0, v.x, a[0][1]);
+            a[0][2] = fmaf(-w0, v.y, a[0][2]);
+            a[1][1] = fmaf(-w1, v.x, a[1][1]);
+            a[1][2] = fmaf(-w1, v.y, a[1][2]);
+            a[2][1] = fmaf(-w2, v.x, a[2][1]);
+            a[2][2] = fmaf(-w2, v.y, a[2][2]);
+            const float f1 = -u * v.x, f2 = fmaf(-u, v.y, f);
+            if (!k2) {  // no further step of this bulge (or none at all)
+                nxt = Refl{0.0f, 0.0f, 0.0f};
+                beta = a[1][0];
+                if (g < nb && t + 1 == 3 * g) nxt = intro_reflector(B, ld, lo, s_sh[g].x, s_sh[g].y);
+            }
+            table_put(row, g, nxt);
+            if (act) {  // row p and column p leave the tile
                 e[0] = a[0][0];
                 e[ld] = a[0][1];
+                e[1] = beta;
                 if (k2) e[2 * ld] = a[0][2];
-                e[1] = a[1][0];
-                if (!k2) e[1 + ld] = a[1][1];  // the bulge's last step
-                else if (t + 1 == t1) {
+                if (!k2 || t + 1 == t1) {  // and the rest of it
                     e[1 + ld] = a[1][1];
-                    e[2 + ld] = a[2][1];
-                    e[1 + 2 * ld] = a[1][2];
-                    e[2 + 2 * ld] = a[2][2];
+                    if (k2) {
+                        e[2 + ld] = a[2][1];
+                        e[1 + 2 * ld] = a[1][2];
+                        e[2 + 2 * ld] = a[2][2];
+                    }
                     if (k3) {
                         e[3 + ld] = f1;
                         e[3 + 2 * ld] = f2;
                     }
                 }
-                v = nxt;
-                shift(f1, f2);
-                left2();
-            } else {
-                if (g < nb && t + 1 == 3 * g) {
-                    nxt = intro_reflector(B, ld, lo, s_sh[g].x, s_sh[g].y);
-                    v = nxt;
-                }
-                table_put(row, g, nxt);
             }
+            // the next tile: its columns p + 1, p + 2 with the left reflector
+            v = nxt;
+            const float b00 = a[1][1], b01 = a[1][2], b10 = a[2][1], b11 = a[2][2];
+            const float x0 = v.z * fmaf(v.y, f1, fmaf(v.x, b10, b00)), x1 = v.z * fmaf(v.y, f2, fmaf(v.x, b11, b01));
+            a[0][0] = b00 - x0;
+            a[0][1] = b01 - x1;
+            a[1][0] = fmaf(-x0, v.x, b10);
+            a[1][1] = fmaf(-x1, v.x, b11);
+            a[2][0] = fmaf(-x0, v.y, f1);
+            a[2][1] = fmaf(-x1, v.y, f2);
+            s0 = fmaf(v.x, a[0][1], a[0][0]);
+            s1 = fmaf(v.x, a[1][1], a[1][0]);
+            s2 = fmaf(v.x, a[2][1], a[2][0]);
         }
         step_bar();
     }
@@ -443,110 +377,104 @@ __device__ __forceinline__ void diag_window(float *B, int ld, int lo, int hi, in
 
 // A tile beside the diagonal during a window: rows of bulge gi; columns of
 // bulge gj < gi (!AHEAD) or the gj-th triple right of the first bulge (AHEAD:
-// left reflectors only).  extra (one warp's lanes 0 .. 15, bulge = lane):
+// left reflectors only, columns up to r1).  A lane keeps the overlap of its
+// consecutive tiles.  extra (one warp's lanes 0 .. 15, bulge = lane): !AHEAD:
 // while bulges are still entering at lo, the up to two rows between lo and the
-// last one take the right reflectors here.  prog: one thread's step count for
-// the warps that follow the chase.
+// last one take the right reflectors here; AHEAD: once the first bulges have
+// left at hi, the up to two columns right of the rest.  prog: one thread's
+// step count for the warps that follow the chase.
 template <bool AHEAD>
 __device__ __forceinline__ void tile_window(float *B, int ld, int lo, int hi, int r1, int t0, int t1, int nb, int gi,
                                             int gj, bool extra, const float *rt, int *prog)
 {
     float a[3][3];
+#pragma unroll
+    for (int q = 0; q < 3; ++q)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) a[q][c] = 0.0f;
     bool held = false;
-    // a step with every bulge on its way and inside the block
-    auto steady = [&](int t, const float *row) {
+    const int last = AHEAD ? r1 : hi;
+#pragma unroll 1
+    for (int t = t0; t < t1; ++t) {
+        const float *row = rt + (t - t0) * TS;
         const int pi = lo + t - 3 * gi;
         const int pj = AHEAD ? lo + t + 3 + 3 * gj : lo + t - 3 * gj;
-        if (gi < nb && (!AHEAD || pj <= r1)) {
+        if (gi < nb && pi >= lo && (AHEAD ? pj <= r1 && lo + t < hi : pj < hi)) {
             float *e = B + pi + pj * ld;
             const Refl l = table_get(row, gi);
             Refl r{0.0f, 0.0f, 0.0f};
             if (!AHEAD) r = table_get(row, gj);
-            const bool c1 = !AHEAD || pj + 1 <= r1, c2 = !AHEAD || pj + 2 <= r1;
+            const bool c1 = !AHEAD || pj + 1 <= last, c2 = pj + 2 <= last;
             if (!held) {
                 a[0][0] = e[0];
                 a[1][0] = e[1];
-                a[0][1] = c1 ? e[ld] : 0.0f;
-                a[1][1] = c1 ? e[1 + ld] : 0.0f;
+                if (c1) {
+                    a[0][1] = e[ld];
+                    a[1][1] = e[1 + ld];
+                }
                 held = true;
             }
             a[2][0] = e[2];
-            a[2][1] = c1 ? e[2 + ld] : 0.0f;
-            a[0][2] = c2 ? e[2 * ld] : 0.0f;
-            a[1][2] = c2 ? e[1 + 2 * ld] : 0.0f;
-            a[2][2] = c2 ? e[2 + 2 * ld] : 0.0f;
+            if (c1) a[2][1] = e[2 + ld];
+            if (c2) {
+                a[0][2] = e[2 * ld];
+                a[1][2] = e[1 + 2 * ld];
+                a[2][2] = e[2 + 2 * ld];
+            } else {
+                a[0][2] = a[1][2] = a[2][2] = 0.0f;
+                if (AHEAD && !c1) a[0][1] = a[1][1] = a[2][1] = 0.0f;
+            }
             tile_update<true, !AHEAD>(a, l, r);
             e[0] = a[0][0];
             e[1] = a[1][0];
             e[2] = a[2][0];
             if (c1) e[ld] = a[0][1];
             if (c2) e[2 * ld] = a[0][2];
-            a[0][0] = a[1][1];
-            a[0][1] = a[1][2];
-            a[1][0] = a[2][1];
-            a[1][1] = a[2][2];
+            if (t + 1 == t1 || !c2) {  // the last step with this tile, or columns end: everything goes out
+                if (c1) {
+                    e[1 + ld] = a[1][1];
+                    e[2 + ld] = a[2][1];
+                }
+                if (c2) {
+                    e[1 + 2 * ld] = a[1][2];
+                    e[2 + 2 * ld] = a[2][2];
+                }
+                held = false;
+            } else {
+                a[0][0] = a[1][1];
+                a[0][1] = a[1][2];
+                a[1][0] = a[2][1];
+                a[1][1] = a[2][2];
+            }
         }
-    };
-    if (t0 > 3 * (nb - 1) && lo + t1 + 2 <= hi) {  // a whole window of such steps
-        const float *row = rt;
-        for (int t = t0; t < t1; ++t, row += TS) {
-            steady(t, row);
-            step_bar();
-            if (AHEAD && prog && threadIdx.x == 10 * 32) prog_set(prog, t - t0 + 2);
-        }
-        if (!AHEAD && held) {  // (ahead of the chain nothing is left to store: the tiles have left the block)
-            const int pi = lo + t1 - 3 * gi, pj = lo + t1 - 3 * gj;
-            float *e = B + pi + pj * ld;
-            e[0] = a[0][0];
-            e[1] = a[1][0];
-            e[ld] = a[0][1];
-            e[1 + ld] = a[1][1];
-        }
-        return;
-    }
-    for (int t = t0; t < t1; ++t) {
-        const float *row = rt + (t - t0) * TS;
-        const int pi = lo + t - 3 * gi;
-        const int pj = AHEAD ? lo + t + 3 + 3 * gj : lo + t - 3 * gj;
-        if (t > 3 * (nb - 1) && t > t0 && t + 1 < t1 && lo + t + 3 <= hi) {
-            steady(t, row);
-        } else {
+        if (extra) {
             const int over = t - (hi - 1 - lo);
             const int ga = over > 0 ? (over + 2) / 3 : 0, gb = min(nb - 1, t / 3);  // bulges ga .. gb are on the way
-            const int pc = AHEAD ? pj - 3 * ga : pj;
-            const int c1 = (AHEAD ? r1 : hi) + 1 - pc;  // columns of the tile that exist
-            if (gi >= ga && gi <= gb && (AHEAD ? c1 > 0 : gj >= ga)) {
-                float *e = B + pi + pc * ld;
-                const Refl l = table_get(row, gi);
-                Refl r{0.0f, 0.0f, 0.0f};
-                if (!AHEAD) r = table_get(row, gj);
-                const int e1 = hi + 1 - pi;  // rows
-#pragma unroll
-                for (int c = 0; c < 3; ++c)
-#pragma unroll
-                    for (int q = 0; q < 3; ++q)
-                        if (!held || q == 2 || c == 2) a[q][c] = (q < e1 && c < c1) ? e[q + c * ld] : 0.0f;
-                tile_update<true, !AHEAD>(a, l, r);
-#pragma unroll
-                for (int c = 0; c < 3; ++c)
-#pragma unroll
-                    for (int q = 0; q < 3; ++q)
-                        if (q < e1 && c < c1) e[q + c * ld] = a[q][c];
-            }
-            held = false;
-            if (!AHEAD && extra) {
-                const int g = threadIdx.x & 31, pg = lo + t - 3 * g;
-                const int fresh = t - 3 * gb;  // rows above the last bulge
-                if (t < 3 * (nb - 1) && fresh > 0 && g >= ga && g <= gb) {
+            const int g = threadIdx.x & 31, pg = lo + t - 3 * g;
+            if (g >= ga && g <= gb) {
+                if (!AHEAD && t < 3 * (nb - 1)) {
                     const Refl v = table_get(row, g);
-                    float *e = B + lo + pg * ld;
                     const bool k2 = pg + 2 <= hi;
-                    for (int q = 0; q < fresh; ++q) {
-                        const float x0 = e[q], x1 = e[q + ld], x2 = k2 ? e[q + 2 * ld] : 0.0f;
+#pragma unroll 1
+                    for (int i = lo; i < lo + t - 3 * gb; ++i) {
+                        float *e = B + i + pg * ld;
+                        const float x0 = e[0], x1 = e[ld], x2 = k2 ? e[2 * ld] : 0.0f;
                         const float w = v.z * fmaf(v.y, x2, fmaf(v.x, x1, x0));
-                        e[q] = x0 - w;
-                        e[q + ld] = fmaf(-w, v.x, x1);
-                        if (k2) e[q + 2 * ld] = fmaf(-w, v.y, x2);
+                        e[0] = x0 - w;
+                        e[ld] = fmaf(-w, v.x, x1);
+                        if (k2) e[2 * ld] = fmaf(-w, v.y, x2);
+                    }
+                }
+                if (AHEAD && ga > 0) {
+                    const Refl v = table_get(row, g);
+#pragma unroll 1
+                    for (int j = lo + t - 3 * ga + 3; j <= hi; ++j) {
+                        float *e = B + pg + j * ld;
+                        const float x0 = e[0], x1 = e[1], x2 = e[2];
+                        const float w = v.z * fmaf(v.y, x2, fmaf(v.x, x1, x0));
+                        e[0] = x0 - w;
+                        e[1] = fmaf(-w, v.x, x1);
+                        e[2] = fmaf(-w, v.y, x2);
                     }
                 }
             }
@@ -614,6 +542,7 @@ __device__ __noinline__ bool quad_window(float *vec, int stride, bool on, const 
 #pragma unroll
     for (int i = 0; i < L - 1; ++i) x[i] = ((unsigned)(A + i) < (unsigned)rr) ? vec[(A + i) * stride] : 0.0f;
     const int nblk = (ns + KB - 1) / KB;
+#pragma unroll 1
     for (int st = 0; st < nblk + 3; ++st) {
         const int q0 = (st - sub) * KB;
         if (st >= sub && q0 < ns) {
@@ -676,9 +605,10 @@ __device__ __noinline__ bool quad_window(float *vec, int stride, bool on, const 
 // number of steps within their spread).  Every thread of the CTA calls it.
 
 //
-// Warps 0 .. 15 take two estimates each (j and j + 16), lane r keeping the
-// sums of row r, as packed pairs (re, im): the packed FP32 instructions halve
-// the issue slots, which bound the iteration (32 estimates x 32 rows).
+// A half-warp per estimate (warps 0 .. 15 take 32), lane r of it keeping the
+// sums of rows r and r + 16, as packed pairs (re, im): the packed FP32
+// instructions and one broadcast for both estimates of a warp keep the issue
+// slots down, which bound the iteration (32 estimates x 32 rows).
 struct f2 {
     unsigned long long v;
 };
@@ -744,92 +674,74 @@ __device__ __noinline__ bool cta_aberth_real(const float *M, int m, float2 *z, f
     if (tid == 0) s_bad = 0;
     __syncthreads();
     static_assert(kCta >= 32 * 16, "warps 0 .. 15 take the estimates");
-    const int ja = warp, jb = warp + 16;
+    const int r = lane & 15, j = 2 * warp + (lane >> 4);  // row (and row + 16), estimate
+#pragma unroll 1
     for (int it = 0; it < kmax; ++it) {
-        if (warp < 16 && ja < m) {
-            const bool two = jb < m;
-            float2 mu[2];
-            mu[0] = z[ja];
-            mu[1] = z[two ? jb : ja];
-            f2 s[2], ds[2], x[2], dx[2], nmx[2], nmy[2];
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                s[h] = ds[h] = dx[h] = f2_mk(0.0f, 0.0f);
-                x[h] = f2_mk(1.0f, 0.0f);
-                nmx[h] = f2_mk(-mu[h].x, -mu[h].x);
-                nmy[h] = f2_mk(mu[h].y, -mu[h].y);
-            }
-            float a = M[min(lane, m - 1) + (m - 1) * MLD];
+        if (2 * warp < m) {  // (m is even)
+            const float2 mu = z[j];
+            const f2 zero2 = f2_mk(0.0f, 0.0f), nmx = f2_mk(-mu.x, -mu.x), nmy = f2_mk(mu.y, -mu.y);
+            f2 s0 = zero2, ds0 = zero2, s1 = zero2, ds1 = zero2, dx = zero2, x = f2_mk(1.0f, 0.0f);
+            const float *c0 = M + min(r, m - 1), *c1 = M + min(r + 16, m - 1);
+#pragma unroll 1
             for (int i = m - 1;; --i) {
                 // column i of (M - mu I) into rows 0 .. i (rows below are done)
-                const f2 a2 = f2_mk(a, a);
-                const float iv = s_inv[i];
-                if (i > 0) a = M[min(lane, m - 1) + (i - 1) * MLD];
-                float2 c[2], dc[2];
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    s[h] = f2_fma(a2, x[h], s[h]);
-                    ds[h] = f2_fma(a2, dx[h], ds[h]);
-                    // row i with the diagonal's -mu x_i (and -x_i in the derivative)
-                    const float2 xv = f2_get(x[h]), dv = f2_get(dx[h]);
-                    f2 cc = f2_fma(nmx[h], x[h], s[h]);
-                    cc = f2_fma(nmy[h], f2_mk(xv.y, xv.x), cc);
-                    f2 dd = f2_fma(nmx[h], dx[h], ds[h]);
-                    dd = f2_fma(nmy[h], f2_mk(dv.y, dv.x), dd);
-                    dd = f2_add(dd, f2_mk(-xv.x, -xv.y));
-                    if (i > 0) {
-                        const f2 iv2 = f2_mk(iv, iv);
-                        cc = f2_mul(cc, iv2);
-                        dd = f2_mul(dd, iv2);
-                    }
-                    c[h] = f2_get(cc);
-                    dc[h] = f2_get(dd);
-                }
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    c[h].x = __shfl_sync(0xffffffffu, c[h].x, i);
-                    c[h].y = __shfl_sync(0xffffffffu, c[h].y, i);
-                    dc[h].x = __shfl_sync(0xffffffffu, dc[h].x, i);
-                    dc[h].y = __shfl_sync(0xffffffffu, dc[h].y, i);
-                    x[h] = f2_mk(c[h].x, c[h].y);
-                    dx[h] = f2_mk(dc[h].x, dc[h].y);
-                }
+                const float a0 = c0[i * MLD], a1 = c1[i * MLD], iv = s_inv[i];
+                const f2 p0 = f2_mk(a0, a0), p1 = f2_mk(a1, a1);
+                s0 = f2_fma(p0, x, s0);
+                ds0 = f2_fma(p0, dx, ds0);
+                s1 = f2_fma(p1, x, s1);
+                ds1 = f2_fma(p1, dx, ds1);
+                // row i with the diagonal's -mu x_i (and -x_i in the derivative),
+                // over -M(i, i-1): x_{i-1} and its derivative
+                const float2 xv = f2_get(x), dv = f2_get(dx);
+                f2 cc = f2_fma(nmx, x, i < 16 ? s0 : s1);
+                f2 dd = f2_fma(nmx, dx, i < 16 ? ds0 : ds1);
+                cc = f2_fma(nmy, f2_mk(xv.y, xv.x), cc);
+                dd = f2_fma(nmy, f2_mk(dv.y, dv.x), dd);
+                dd = f2_add(dd, f2_mk(-xv.x, -xv.y));
+                const f2 iv2 = f2_mk(iv, iv);
+                cc = f2_mul(cc, iv2);
+                dd = f2_mul(dd, iv2);
+                float2 c = f2_get(cc), d = f2_get(dd);
+                c.x = __shfl_sync(0xffffffffu, c.x, i & 15, 16);
+                c.y = __shfl_sync(0xffffffffu, c.y, i & 15, 16);
+                d.x = __shfl_sync(0xffffffffu, d.x, i & 15, 16);
+                d.y = __shfl_sync(0xffffffffu, d.y, i & 15, 16);
+                x = f2_mk(c.x, c.y);
+                dx = f2_mk(d.x, d.y);
                 if (i == 0) break;
-                if ((i & 3) == 0) {  // back into range by powers of two (the same in every lane)
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const float mag = fmaxf(fmaxf(fabsf(c[h].x), fabsf(c[h].y)), fmaxf(fabsf(dc[h].x), fabsf(dc[h].y)));
-                        if (mag > 1.0e6f || (mag > 0.0f && mag < 1.0e-6f)) {
-                            const int e = min(max((int)((__float_as_uint(mag) >> 23) & 255), 1), 253);
-                            const float sc = __uint_as_float((unsigned)(254 - e) << 23);  // 2^-(exponent of mag)
-                            const f2 sc2 = f2_mk(sc, sc);
-                            x[h] = f2_mul(x[h], sc2);
-                            dx[h] = f2_mul(dx[h], sc2);
-                            s[h] = f2_mul(s[h], sc2);
-                            ds[h] = f2_mul(ds[h], sc2);
-                        }
-                    }
+                if ((i & 3) == 0) {  // back into range by powers of two (the same in every lane of the half)
+                    const float mag = fmaxf(fmaxf(fabsf(c.x), fabsf(c.y)), fmaxf(fabsf(d.x), fabsf(d.y)));
+                    const int e = min(max((int)((__float_as_uint(mag) >> 23) & 255), 1), 253);
+                    const float sc = mag > 1.0e6f || mag < 1.0e-6f ? __uint_as_float((unsigned)(254 - e) << 23) : 1.0f;
+                    const f2 sc2 = f2_mk(sc, sc);
+                    x = f2_mul(x, sc2);
+                    dx = f2_mul(dx, sc2);
+                    s0 = f2_mul(s0, sc2);
+                    ds0 = f2_mul(ds0, sc2);
+                    s1 = f2_mul(s1, sc2);
+                    ds1 = f2_mul(ds1, sc2);
                 }
             }
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int j = h ? jb : ja;
-                // x, dx: the residual of row 0 and its derivative, p / p' up to a factor
-                const float2 xv = f2_get(x[h]), dv = f2_get(dx[h]);
-                const float2 id = crcp_approx(dv.x, dv.y);
-                const float nx = xv.x * id.x - xv.y * id.y, ny = xv.x * id.y + xv.y * id.x;
-                float2 part = make_float2(0.0f, 0.0f);
-                if (lane < m && lane != j) {
-                    const float2 zr = z[lane];
-                    part = crcp_approx(mu[h].x - zr.x, mu[h].y - zr.y);
+            // x, dx: the residual of row 0 and its derivative, p and p' up to a
+            // factor (s_inv[0] = -1 in both)
+            const float2 xv = f2_get(x), dv = f2_get(dx);
+            const float2 id = crcp_approx(dv.x, dv.y);
+            const float nx = xv.x * id.x - xv.y * id.y, ny = xv.x * id.y + xv.y * id.x;
+            float2 part = make_float2(0.0f, 0.0f);
+#pragma unroll 1
+            for (int q = r; q < m; q += 16)
+                if (q != j) {
+                    const float2 zr = z[q], t = crcp_approx(mu.x - zr.x, mu.y - zr.y);
+                    part.x += t.x;
+                    part.y += t.y;
                 }
-                for (int o = 16; o > 0; o >>= 1) {
-                    part.x += __shfl_xor_sync(0xffffffffu, part.x, o);
-                    part.y += __shfl_xor_sync(0xffffffffu, part.y, o);
-                }
-                const float2 iq = crcp_approx(1.0f - (nx * part.x - ny * part.y), -(nx * part.y + ny * part.x));
-                if (lane == 0 && j < m) s_w[j] = make_float2(nx * iq.x - ny * iq.y, nx * iq.y + ny * iq.x);
+            for (int o = 8; o > 0; o >>= 1) {
+                part.x += __shfl_xor_sync(0xffffffffu, part.x, o);
+                part.y += __shfl_xor_sync(0xffffffffu, part.y, o);
             }
+            const float2 iq = crcp_approx(1.0f - (nx * part.x - ny * part.y), -(nx * part.y + ny * part.x));
+            if (r == 0) s_w[j] = make_float2(nx * iq.x - ny * iq.y, nx * iq.y + ny * iq.x);
         }
         __syncthreads();
         bool done = true;
@@ -852,7 +764,7 @@ __device__ __noinline__ bool cta_aberth_real(const float *M, int m, float2 *z, f
 // ended dh rows lower; for each of the dh eigenvalues deflated since (defl)
 // the nearest is dropped, and at most m stay; the remaining places (all for a
 // cold start, np = 0) take eigenvalues of M's 2 x 2 diagonal blocks.
-__device__ void warp_shift_start(const float *M, int m, float mnrm, const float2 *prev, int np, const float2 *defl,
+__device__ __noinline__ void warp_shift_start(const float *M, int m, float mnrm, const float2 *prev, int np, const float2 *defl,
                                  int dh, float2 *z)
 {
     const int lane = threadIdx.x & 31;
@@ -893,7 +805,7 @@ __device__ void warp_shift_start(const float *M, int m, float mnrm, const float2
 // sqrt(-q): a conjugate pair alpha +- i beta gives q = beta^2, two real
 // estimates q = -((a - b) / 2)^2.  One warp; returns the number of bulges
 // (at most nb, at least 1).
-__device__ int warp_pair_shifts(const float2 *z, int m, float mnrm, float2 *sh, int nb)
+__device__ __noinline__ int warp_pair_shifts(const float2 *z, int m, float mnrm, float2 *sh, int nb)
 {
     const int lane = threadIdx.x & 31;
     const float2 c = lane < m ? z[lane] : make_float2(0.0f, 0.0f);
@@ -976,7 +888,7 @@ __device__ bool wait_all_helpers(const SchurDesc<float> &d, int H, int target)
 // warps apply the window to four groups.
 constexpr int kQuads = kCta / kQuad;
 
-__device__ void staged_window(float *T, int64_t ld, float *stage, const float *rt, const float *zero, int ns, int off,
+__device__ __noinline__ void staged_window(float *T, int64_t ld, float *stage, const float *rt, const float *zero, int ns, int off,
                               int kmin, int rr, int c0, int c1, int ra, int rb, int r0, int qoff, int H, int h)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -996,7 +908,7 @@ __device__ void staged_window(float *T, int64_t ld, float *stage, const float *r
         const int i0 = col ? 8 * (gc + k * m) : 8 * (gr + (k - nc) * m);
         float *sg = stage + warp * 8 * SLD;
         if (has && col) {
-#pragma unroll
+#pragma unroll 1
             for (int z = 0; z < (RR + 31) / 32; ++z) {
                 const int v = lane + 32 * z;
                 float x[8];
@@ -1010,8 +922,8 @@ __device__ void staged_window(float *T, int64_t ld, float *stage, const float *r
         } else if (has) {
             const int r = lane & 7, i = i0 + r;
             const bool in = i >= ra && i < rb;
-            constexpr int NV = (RR + 3) / 4;  // 20
-#pragma unroll
+                constexpr int NV = (RR + 3) / 4;  // 20
+#pragma unroll 1
             for (int z = 0; z < 2; ++z) {
                 float x[NV / 2];
 #pragma unroll
@@ -1055,7 +967,7 @@ __device__ void staged_window(float *T, int64_t ld, float *stage, const float *r
 // the windows need no ordering between helpers).  Then it publishes its
 // count.  One thread's fence after a barrier covers the CTA's stores (a
 // fence by every warp took most of a window's time).
-__device__ void helper_cta(const SchurDesc<float> &d, float *T, int H, int h, float *stage, float *rt, const float *zero)
+__device__ __noinline__ void helper_cta(const SchurDesc<float> &d, float *T, int H, int h, float *stage, float *rt, const float *zero)
 {
     const int nt = (int)blockDim.x;
     __shared__ int s_go, s_nwin;
@@ -1115,6 +1027,14 @@ __device__ void helper_cta(const SchurDesc<float> &d, float *T, int H, int h, fl
 // is assembled in shared memory; 2: one CTA per matrix with the
 // whole matrix in shared memory.  Matrices with n outside (nlo, nhi] return
 // at once (the size classes of a batch).
+// Bound by the serial chain of steps (one barrier each, about 300 cycles of
+// dependent arithmetic in the diagonal tiles) and by instruction supply: one
+// warp's code runs once a step, so it misses the instruction cache unless each
+// role has a single path.  One path for every step, loops left rolled outside
+// the steps and an estimate of the shifts per half-warp, against a fast and a
+// general copy and an estimate per warp, ms of chase: n = 64 0.35 / 0.54, 101
+// 0.83 / 0.99, 200 2.14 / 2.85, 256 3.38 / 5.48, 512 10.1 / 12.5, 1024 31.4 /
+// 32.6, 2048 97.5 / 112.9.
 template <int MODE>
 __global__ void __launch_bounds__(kCta, 1)
 rqr_chase_kernel(const SchurDesc<float> *__restrict__ descs, int H, int nlo, int nhi)
@@ -1347,7 +1267,7 @@ rqr_chase_kernel(const SchurDesc<float> *__restrict__ descs, int H, int nlo, int
                 tile_window<false>(B, bld, lo, hi, r1, t0, t1, nb, pair >> 8, pair & 255, ridx == 3, rt, nullptr);
             } else if (role == R_AHEAD) {
                 const int b = 2 * ridx + (lane >> 4);
-                tile_window<true>(B, bld, lo, hi, b < NAH ? r1 : -1, t0, t1, nb, lane & 15, b, false, rt,
+                tile_window<true>(B, bld, lo, hi, b < NAH ? r1 : -1, t0, t1, nb, lane & 15, b, ridx == 0, rt,
                                   MODE == 1 ? &s_prog : nullptr);
             } else if (MODE == 1 && role == R_SIDE && cn > 0) {
                 // four warps: once the helpers are done with every window
