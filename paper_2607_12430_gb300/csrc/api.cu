@@ -331,10 +331,6 @@ static int read_scalars(sqrtm_handle_t h, const Scalars &s, double *norm, double
 static bool is_bitwise_symmetric(sqrtm_handle_t h, const double *dA, int64_t n, int64_t lda,
                                  int *flag_dev, int *rc);
 
-// smallest n whose general-path residual uses the split-BF16 tensor-core
-// products (below it the FP64 CUDA-core product is as fast)
-static constexpr int64_t kGenSplitMinN = 512;
-
 // ---------------------------------------------------------------------------
 // general path (Algorithm 2) in storage precision R; refine = false gives the
 // plain Schur method.  root = 3 gives the principal cube root (Sec. 4, p = 3)
@@ -579,6 +575,9 @@ static int general_path(sqrtm_handle_t h, const double *dA, int64_t n, int64_t l
             } else if (use_gsplit) {
                 SQM_CU(launch_residual_gen_split(dA, lda, dX, ldx, (int)n, e, Rhat, (int)n, gRacc, gXT, gDa, gDb, gRhoA,
                                                  gRhoB, sc.partials, &np, sc.st_solve, s));
+            } else if (sizeof(R) == sizeof(float) && n > kXsplitMinN && n < kGenSplitMinN &&
+                       !(o.precision & SQRTM_PREC_RESID_FP64)) {
+                SQM_CU(launch_xsplit_residual(dA, lda, dX, ldx, (int)n, e, norm_a, Rhat, (int)n, sc.partials, &np, s));
             } else {
                 SQM_CU(launch_residual_f64(dA, lda, dX, ldx, (int)n, e, Rhat, (int)n, sc.partials, &np, s));
             }

@@ -459,6 +459,7 @@ struct Pipe {
     BLayout<float> L;
     const int *nord;  // sizes in batch order (host)
     int B, Bg, nmax, blks;
+    bool resid_fp64;  // FP64 products in the residual asked for
     cudaStream_t body_stream;
 };
 
@@ -471,7 +472,8 @@ cudaError_t enqueue_refine_body(void *p, cudaStream_t s, cudaGraphConditionalHan
     cudaError_t err;
     // R = (A - X X) 4^-e and ||R||_F, the per-matrix test (counting the
     // matrices that go on), R~ = Q^H Rhat Q, S Y + Y S = R~, X += 2^e Re(Q Y Q^H)
-    if ((err = launch_residual_batched(L.rj, B, nm, s))) return err;
+    if ((err = c->resid_fp64 ? launch_residual_batched(L.rj, B, nm, s) : launch_xsplit_residual_batched(L.rj, B, nm, s)))
+        return err;
     bdecide_kernel<<<cdiv_i(B, 128), 128, 0, s>>>(L.st, B, L.prm); count_launch();
     if ((err = launch_cgemm_batched<R>(OP_N, OP_N, true, EPI_STORE, L.gj + 2 * B, B, nm, s))) return err;
     if ((err = launch_cgemm_batched<R>(OP_H, OP_N, false, EPI_STORE, L.gj + 3 * B, B, nm, s))) return err;
@@ -652,7 +654,7 @@ int batched_general(sqrtm_handle_t h, const int *idx, int count, const double *c
     ResJob *hrj = (ResJob *)host(L.rj);
     BInput *hin = (BInput *)host(L.in);
     BParams *hprm = (BParams *)host(L.prm);
-    const bool fixed = o.steps >= 0;
+    const bool fixed = o.steps >= 0, resid_fp64 = (o.precision & SQRTM_PREC_RESID_FP64) != 0;
     hprm->tol = o.tol;
     hprm->fixed = fixed;
     hprm->max_corr = fixed ? o.steps : o.maxit + 1;
@@ -695,10 +697,10 @@ int batched_general(sqrtm_handle_t h, const int *idx, int count, const double *c
         hgj[3 * B + i] = GemmJob<R>{Q, W, Rt, nullptr, 0, &q->e, &q->active, (int)nm};
         hgj[4 * B + i] = GemmJob<R>{Q, Rt, W, nullptr, 0, &q->e, &q->active, (int)nm};
         hgj[5 * B + i] = GemmJob<R>{W, Q, nullptr, dX[m], ldx[m], &q->e, &q->active, (int)nm};
-        hrj[i] = ResJob{dA[m], lda[m], dX[m], ldx[m], Rhat, partials, &q->e, &q->active, (int)nm};
+        hrj[i] = ResJob{dA[m], lda[m], dX[m], ldx[m], Rhat, partials, &q->e, &q->active, &q->norm_a, (int)nm};
         BState *hq = (BState *)host(q);
         hq->partials = partials;
-        hq->np = (int)(nt * nt);
+        hq->np = resid_fp64 ? residual_f64_parts((int)nm) : xsplit_parts((int)nm);
     }
     SQM_CU(cudaMemcpyAsync(h->bws.p, hdr.data(), L.hdr_bytes, cudaMemcpyHostToDevice, s));
     if (!h->body_stream) SQM_CU(cudaStreamCreateWithFlags(&h->body_stream, cudaStreamNonBlocking));
@@ -707,10 +709,11 @@ int batched_general(sqrtm_handle_t h, const int *idx, int count, const double *c
     // one graph for the whole call, keyed by the sizes and kinds in batch
     // order and the block size (its launches take every pointer from the
     // header just copied)
-    Pipe pipe{L, nord.data(), B, Bg, nmax, o.blks, h->body_stream};
+    Pipe pipe{L, nord.data(), B, Bg, nmax, o.blks, resid_fp64, h->body_stream};
     uint64_t sig = 1469598103934665603ull;
     sig = fnv(sig, (uint64_t)Bg);
     sig = fnv(sig, (uint64_t)o.blks);
+    sig = fnv(sig, (uint64_t)resid_fp64);
     for (int i = 0; i < B; ++i) sig = fnv(sig, (uint64_t)nord[i]);
     if (run_graph(h, 400, L.desc, nmax, B, enqueue_pipeline, &pipe, sig)) return 7;
     BState *hst = (BState *)h->bpin;

@@ -108,6 +108,7 @@ struct ResJob {
     double *partials;
     const int *e;
     const int *active;
+    const double *norm_a;  // ||A||_F
     int n;
 };
 template <class R>
@@ -119,6 +120,19 @@ template <class R>
 cudaError_t launch_cgemm_batched(int opA, int opB, bool a_real, int epi, const GemmJob<R> *jobs, int batch, int nmax,
                                  cudaStream_t s);
 cudaError_t launch_residual_batched(const ResJob *jobs, int batch, int nmax, cudaStream_t s);
+// the same residuals from exact split-BF16 tensor-core products (xsplit.cu)
+// where these are as accurate for a matrix of norm norm_a (FP64 ones where not),
+// xsplit_parts(n) <= residual_f64_parts(n) partial sums each
+int xsplit_parts(int n);
+// The general residual takes FP64 products up to n = kXsplitMinN, xsplit.cu's
+// kernel from there and tc_split.cu's (digits in global memory, TMA) from n =
+// kGenSplitMinN on.  xsplit fills at most the 152 SMs once up to n = 1024 (128
+// tiles).
+constexpr int kXsplitMinN = 32;
+constexpr int64_t kGenSplitMinN = 1025;
+cudaError_t launch_xsplit_residual(const double *A, int64_t lda, const double *X, int64_t ldx, int n, int e,
+                                   double norm_a, float *Rhat, int ldr, double *partials, int *nparts, cudaStream_t s);
+cudaError_t launch_xsplit_residual_batched(const ResJob *jobs, int batch, int nmax, cudaStream_t s);
 
 // ---- scaling / norms (scale.cu) ----
 // Deterministic ||A||_F: partials[nblk] then finalize; writes norm and e, the

@@ -326,8 +326,18 @@ extern "C" int sqrtm_step_residual_split(sqrtm_handle_t h, const double *dA, int
     int *rhoA = c.take<int>(n);
     int *rhoB = c.take<int>(n);
     int np = 0;
-    if (launch_residual_gen_split(dA, lda, dX, ldx, (int)n, e, dRhat, (int)n, Racc, XT, da, db, rhoA, rhoB,
-                                  ss.dscal + 2, &np, ss.iscal + 1, h->stream)) return 7;
+    // the solver's rule: digits formed in the product's kernel below
+    // kGenSplitMinN, where they are accurate for ||A||
+    if (n < kGenSplitMinN) {
+        double nrm;
+        if (launch_norm_scale(dA, n, lda, ss.dscal + 2, (int)n, ss.dscal, ss.iscal, h->stream) ||
+            fetch(h, &nrm, ss.dscal, sizeof(double)) ||
+            launch_xsplit_residual(dA, lda, dX, ldx, (int)n, e, nrm, dRhat, (int)n, ss.dscal + 2, &np, h->stream))
+            return 7;
+    } else if (launch_residual_gen_split(dA, lda, dX, ldx, (int)n, e, dRhat, (int)n, Racc, XT, da, db, rhoA, rhoB,
+                                         ss.dscal + 2, &np, ss.iscal + 1, h->stream)) {
+        return 7;
+    }
     if (launch_sum_partials(ss.dscal + 2, np, ss.dscal + 1, h->stream)) return 7;
     double rn;
     int st = 0;
