@@ -336,8 +336,8 @@ SQRTM_API int sqrtm_mixed_batched(sqrtm_handle_t handle, int batch, const double
 
 /* Phase times of the last batched-path graph on this handle (diagnostic,
  * device clock, ms): [0] norms, scaling and Hessenberg reductions, [1] QR
- * rounds of the general members, [2] Jacobi decompositions of the
- * symmetric members, [3] triangular square roots and X_0, [4] refinement
+ * rounds of the general members, [2] what is left then of the symmetric
+ * members' Jacobi decompositions, which run beside [0] and [1], [3] triangular square roots and X_0, [4] refinement
  * loop.  Copies min(cap, 5) values into ms (HOST), the number of matrices
  * the batched path took into *count and how many of them took Algorithm 2
  * into *general (either may be NULL).  Returns 5, or -1 / -2 (NULL handle /

@@ -460,7 +460,8 @@ struct Pipe {
     const int *nord;  // sizes in batch order (host)
     int B, Bg, nmax, blks;
     bool resid_fp64;  // FP64 products in the residual asked for
-    cudaStream_t body_stream;
+    cudaStream_t body_stream, side;
+    const cudaEvent_t *ev;  // fork and join of the side branch
 };
 
 cudaError_t enqueue_refine_body(void *p, cudaStream_t s, cudaGraphConditionalHandle cond)
@@ -503,6 +504,23 @@ cudaError_t enqueue_pipeline(void *p, cudaStream_t s)
     bnorm_kernel<<<B, kBNormThreads, 0, s>>>(L.in, L.st); count_launch();
     bcast_kernel<R><<<dim3(std::max(1, std::min(64, nmax * nmax / 1024)), B), 256, 0, s>>>(L.in, L.st, L.desc);
     count_launch();
+    // symmetric members: Jacobi, V in global memory above kJacVsmemMaxN, on a
+    // branch beside the general members' stages (one CTA per matrix and a serial
+    // chain of rotations: alone it left most SMs idle, 1.4 ms of a batch of 48's
+    // 5.0 ms and of one of 2048's 130; joined before the triangular square root)
+    if (B > Bg && ((err = cudaEventRecord(c->ev[0], s)) || (err = cudaStreamWaitEvent(c->side, c->ev[0], 0)))) return err;
+    for (int i0 = Bg; i0 < B;) {
+        const bool vs = c->nord[i0] <= kJacVsmemMaxN;
+        int i1 = i0;
+        while (i1 < B && (c->nord[i1] <= kJacVsmemMaxN) == vs) ++i1;
+        const size_t smem = jac_smem_bytes(c->nord[i0], vs);
+        if (vs) bjacobi_kernel<true><<<i1 - i0, kJacThreads, smem, c->side>>>(L.jj + i0);
+        else bjacobi_kernel<false><<<i1 - i0, kJacThreads, smem, c->side>>>(L.jj + i0);
+        count_launch();
+        if ((err = cudaGetLastError())) return err;
+        i0 = i1;
+    }
+    if (B > Bg && (err = cudaEventRecord(c->ev[1], c->side))) return err;
     // general members: Hessenberg reduction (one cluster per matrix, one
     // launch per size class; the per-column kernels beyond the cluster
     // kernel's sizes), then the QR rounds on the device
@@ -524,18 +542,7 @@ cudaError_t enqueue_pipeline(void *p, cudaStream_t s)
                                                      c->body_stream)))
         return err;
     bstamp_kernel<<<1, 1, 0, s>>>(L.stamps, 2); count_launch();
-    // symmetric members: Jacobi, V in global memory above kJacVsmemMaxN
-    for (int i0 = Bg; i0 < B;) {
-        const bool vs = c->nord[i0] <= kJacVsmemMaxN;
-        int i1 = i0;
-        while (i1 < B && (c->nord[i1] <= kJacVsmemMaxN) == vs) ++i1;
-        const size_t smem = jac_smem_bytes(c->nord[i0], vs);
-        if (vs) bjacobi_kernel<true><<<i1 - i0, kJacThreads, smem, s>>>(L.jj + i0);
-        else bjacobi_kernel<false><<<i1 - i0, kJacThreads, smem, s>>>(L.jj + i0);
-        count_launch();
-        if ((err = cudaGetLastError())) return err;
-        i0 = i1;
-    }
+    if (B > Bg && (err = cudaStreamWaitEvent(s, c->ev[1], 0))) return err;
     bstamp_kernel<<<1, 1, 0, s>>>(L.stamps, 3); count_launch();
     if ((err = launch_trisqrt_batched<R>(L.tri, B, nmax, c->blks, s))) return err;
     bfold_kernel<<<cdiv_i(B, 128), 128, 0, s>>>(L.st, B); count_launch();
@@ -709,7 +716,7 @@ int batched_general(sqrtm_handle_t h, const int *idx, int count, const double *c
     // one graph for the whole call, keyed by the sizes and kinds in batch
     // order and the block size (its launches take every pointer from the
     // header just copied)
-    Pipe pipe{L, nord.data(), B, Bg, nmax, o.blks, resid_fp64, h->body_stream};
+    Pipe pipe{L, nord.data(), B, Bg, nmax, o.blks, resid_fp64, h->body_stream, h->side, h->qev};
     uint64_t sig = 1469598103934665603ull;
     sig = fnv(sig, (uint64_t)Bg);
     sig = fnv(sig, (uint64_t)o.blks);
