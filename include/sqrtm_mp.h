@@ -77,7 +77,7 @@ enum { SQRTM_KIND_AUTO = 0, SQRTM_KIND_GENERAL = 1, SQRTM_KIND_SPD = 2, SQRTM_KI
  * summed in FP64 (error-free splitting; the terms left out are below
  * n 2^(rho_i + rho_j - 56), 2^rho_i bounding row i of X, i.e. within the
  * FP64 product's own error bound).  The general path's residual (Algorithm
- * 2, step 4) of a real iterate of the FP32 method, alone or in a batch, does
+ * 2, step 4) of the FP32 method, alone or in a batch, real or complex, does
  * the same from n = 33 on, with the digit slices of the rows of X against
  * those of its columns; up to n = 1024 parts of the product where the digits
  * would be less accurate than FP64 (graded or far from normal X) are formed
@@ -149,7 +149,8 @@ typedef struct {
  *   blks          block size of the triangular square root and Sylvester
  *                 solvers, 1..32 (used when opts->blks == 0);
  *   qr_helpers    helper CTAs of the cooperative QR chase: 0 (chase CTA
- *                 alone), 1..24, or -1 (built-in rule: 8, 16 from n = 1024);
+ *                 alone), 1..24, or -1 (built-in rule: max(8, min(64, n/32))
+ *                 for real input, 8 or from n = 1024 16 for complex);
  *   batched       sqrtm_mixed_batched: 1 sends matrices of these sizes
  *                 through the batched general path, 0 through per-matrix
  *                 calls on worker streams;

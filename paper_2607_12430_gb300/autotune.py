@@ -11,7 +11,7 @@ the SPD path):
   wavefront (Algorithm 1's recursion cut-off; Sec. 5 uses 32): candidates
   8, 16, 32, on sqrtm_mixed with a fixed number of corrections;
 * qr_helpers -- the helper CTAs of the cooperative QR chase (n >= 256):
-  0, 8, 16;
+  the built-in rule (-1), 0, 8, 16;
 * spd_precision -- FP32 or split-TF32 transforms of Algorithm 3, the faster
   one among those whose forward error against the FP64 method on the same
   GPU, after SPD_STEPS corrections (the stopping test nullified, as in the
@@ -36,7 +36,7 @@ import os
 import numpy as np
 
 BLKS_CANDIDATES = (8, 16, 32)
-HELPER_CANDIDATES = (0, 8, 16)
+HELPER_CANDIDATES = (-1, 0, 8, 16)
 CUTOFF_CANDIDATES = (0, 256, 512)
 SPD_TARGET = 1e-13
 SPD_STEPS = 4  # corrections of the SPD accuracy runs (the protocol of Sec. 5.1: the test nullified)

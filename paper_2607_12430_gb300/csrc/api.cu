@@ -557,6 +557,9 @@ static int general_path(sqrtm_handle_t h, const double *dA, int64_t n, int64_t l
     const double norm_as = ldexp(norm_a, -root * e);
     const bool fixed = o.steps >= 0;
     const int max_corr = fixed ? o.steps : o.maxit + 1;
+    // digit products of the residual formed in the product's kernel
+    const bool xsplit = sizeof(R) == sizeof(float) && n > kXsplitMinN && n < kGenSplitMinN &&
+                        !(o.precision & SQRTM_PREC_RESID_FP64);
     int status = 0, applied = 0, grew = 0;
     double prev = INFINITY;
     for (int k = 0;; ++k) {
@@ -567,17 +570,24 @@ static int general_path(sqrtm_handle_t h, const double *dA, int64_t n, int64_t l
             if (root == 3) {
                 SQM_CU(launch_rgemm<double>(0, 0, (int)n, (int)n, (int)n, dX, (int)ldx, dX, (int)ldx, RG_STORE, XX,
                                             (int)n, nullptr, nullptr, 0, 0.0, s));
-                SQM_CU(launch_residual_f64_ab(dA, lda, dX, ldx, XX, n, (int)n, 3 * e, Rhat, (int)n, sc.partials,
-                                              &np, s));
+                if (xsplit)
+                    SQM_CU(launch_xsplit_residual(dA, lda, dX, ldx, XX, n, (int)n, 3 * e, norm_a, Rhat, (int)n,
+                                                  sc.partials, &np, s));
+                else
+                    SQM_CU(launch_residual_f64_ab(dA, lda, dX, ldx, XX, n, (int)n, 3 * e, Rhat, (int)n, sc.partials,
+                                                  &np, s));
+            } else if (cin && xsplit) {
+                SQM_CU(launch_xsplit_zresidual(dA, lda, dX, ldx, (int)n, 2 * e, norm_a, (cplx<float> *)Rhat, (int)n,
+                                               sc.partials, &np, s));
             } else if (cin) {
                 SQM_CU(launch_zresidual_f64(dA, lda, dX, ldx, (int)n, e, (cplx<float> *)Rhat, (int)n, sc.partials, &np,
                                             s));
             } else if (use_gsplit) {
                 SQM_CU(launch_residual_gen_split(dA, lda, dX, ldx, (int)n, e, Rhat, (int)n, gRacc, gXT, gDa, gDb, gRhoA,
                                                  gRhoB, sc.partials, &np, sc.st_solve, s));
-            } else if (sizeof(R) == sizeof(float) && n > kXsplitMinN && n < kGenSplitMinN &&
-                       !(o.precision & SQRTM_PREC_RESID_FP64)) {
-                SQM_CU(launch_xsplit_residual(dA, lda, dX, ldx, (int)n, e, norm_a, Rhat, (int)n, sc.partials, &np, s));
+            } else if (xsplit) {
+                SQM_CU(launch_xsplit_residual(dA, lda, dX, ldx, dX, ldx, (int)n, 2 * e, norm_a, Rhat, (int)n,
+                                              sc.partials, &np, s));
             } else {
                 SQM_CU(launch_residual_f64(dA, lda, dX, ldx, (int)n, e, Rhat, (int)n, sc.partials, &np, s));
             }

@@ -130,8 +130,13 @@ int xsplit_parts(int n);
 // tiles).
 constexpr int kXsplitMinN = 32;
 constexpr int64_t kGenSplitMinN = 1025;
-cudaError_t launch_xsplit_residual(const double *A, int64_t lda, const double *X, int64_t ldx, int n, int e,
-                                   double norm_a, float *Rhat, int ldr, double *partials, int *nparts, cudaStream_t s);
+// R = (A - X Y) 2^-shift; complex: Y = X, 2 xsplit_parts(n) partial sums
+cudaError_t launch_xsplit_residual(const double *A, int64_t lda, const double *X, int64_t ldx, const double *Y,
+                                   int64_t ldy, int n, int shift, double norm_a, float *Rhat, int ldr, double *partials,
+                                   int *nparts, cudaStream_t s);
+cudaError_t launch_xsplit_zresidual(const double *A, int64_t lda, const double *X, int64_t ldx, int n, int shift,
+                                    double norm_a, cplx<float> *Rhat, int ldr, double *partials, int *nparts,
+                                    cudaStream_t s);
 cudaError_t launch_xsplit_residual_batched(const ResJob *jobs, int batch, int nmax, cudaStream_t s);
 
 // ---- scaling / norms (scale.cu) ----

@@ -332,7 +332,7 @@ extern "C" int sqrtm_step_residual_split(sqrtm_handle_t h, const double *dA, int
         double nrm;
         if (launch_norm_scale(dA, n, lda, ss.dscal + 2, (int)n, ss.dscal, ss.iscal, h->stream) ||
             fetch(h, &nrm, ss.dscal, sizeof(double)) ||
-            launch_xsplit_residual(dA, lda, dX, ldx, (int)n, e, nrm, dRhat, (int)n, ss.dscal + 2, &np, h->stream))
+            launch_xsplit_residual(dA, lda, dX, ldx, dX, ldx, (int)n, 2 * e, nrm, dRhat, (int)n, ss.dscal + 2, &np, h->stream))
             return 7;
     } else if (launch_residual_gen_split(dA, lda, dX, ldx, (int)n, e, dRhat, (int)n, Racc, XT, da, db, rhoA, rhoB,
                                          ss.dscal + 2, &np, ss.iscal + 1, h->stream)) {

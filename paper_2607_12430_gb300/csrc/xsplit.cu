@@ -1,5 +1,6 @@
-// xsplit.cu -- the FP64 residual R = (A - X Y) 4^-e of small and middling
-// matrices, one or a batch, the product from exact digit products on the BF16
+// xsplit.cu -- the FP64 residual R = (A - X Y) 2^-s of small and middling
+// matrices, one, a batch or one complex one (Y = X, or X X for the cube root),
+// the product from exact digit products on the BF16
 // tensor cores (the error-free splitting of Ozaki, Ogita, Oishi and Rump,
 // Numer. Algorithms 59 (2012)), with the digits formed in the kernel.
 //
@@ -38,6 +39,9 @@
 // that are not finite) and for n <= 32, where there is less to do than the
 // digits cost.
 //
+// A complex product is two real ones with 2 n terms each, the imaginary parts of
+// a row after its real ones: Re = [Xr, -Xi] [Yr; Yi], Im = [Xr, Xi] [Yi; Yr].
+//
 // A tile of a matrix of n = 256 takes about 150 k cycles: 51 k to form the
 // digits, 52 k in the products (89 cycles each; an M = 128, N = 64 product reads
 // 6 KB of shared memory), 33 k in the FP64 units at the end, the rest in the
@@ -46,6 +50,9 @@
 // 316, 512 182 / 600 against FP64 products; against tc_split.cu's kernels 512
 // 182 / 313, 800 253 / 416, 1024 305 / 461 (1025).  Three residuals of a batch of
 // 2048 matrices of 16 to 256 rows: 13 ms, 60 with FP64 products.
+// Refinement of a complex matrix with these and with FP64 products, ms: n = 40
+// 0.48 / 0.95, 101 1.04 / 2.17, 301 2.95 / 6.07; cube root (one of its two
+// products) n = 200 3.76 / 4.26.
 #include <cuda_bf16.h>
 
 #include "internal.h"
@@ -184,6 +191,9 @@ __device__ __forceinline__ bool digits_accurate(const int *ri, const int *sj, in
     return (double)(mr + mc) + 0.5 * (double)log2f(sr * sc * tiles) <= 7.0 + log2(norm_a);
 }
 
+// CPLX: complex A, X, Y and Rhat (interleaved), part blockIdx.z (0 real, 1
+// imaginary) of R; leading dimensions in elements
+template <bool CPLX>
 __global__ void __launch_bounds__(XT, 1)
 xsplit_residual_kernel(XArgs a, const ResJob *__restrict__ jobs)
 {
@@ -204,7 +214,9 @@ xsplit_residual_kernel(XArgs a, const ResJob *__restrict__ jobs)
     }
     const int n = a.n;
     if (m0 >= n || n0 >= n) return;
-    const int part = blockIdx.x + blockIdx.y * cdiv_i(n, XM);
+    constexpr int ES = CPLX ? 2 : 1;  // doubles per element
+    const int im = CPLX ? (int)blockIdx.z : 0;
+    const int part = blockIdx.x + (blockIdx.y + im * cdiv_i(n, XN)) * cdiv_i(n, XM);
     unsigned char *sA = (unsigned char *)(((uintptr_t)smraw + 1023) & ~(uintptr_t)1023);
     unsigned char *sB = sA + XS * XA_BYTES;
     // the scaling exponents of the tile's rows of X and columns of Y
@@ -212,17 +224,20 @@ xsplit_residual_kernel(XArgs a, const ResJob *__restrict__ jobs)
         const int row = m0 + (tid & (XM - 1)), g = tid / XM;
         unsigned mx = 0;
         if (row < n) {
-            const double *x = a.X + row;
+            const double *x = a.X + ES * row;
 #pragma unroll 8
-            for (int k = g; k < n; k += XT / XM) mx = max(mx, (unsigned)__double2hiint(x[(int64_t)k * a.ldx]) & 0x7FFFFFFFu);
+            for (int k = g; k < n; k += XT / XM)
+#pragma unroll
+                for (int p = 0; p < ES; ++p)
+                    mx = max(mx, (unsigned)__double2hiint(x[ES * (int64_t)k * a.ldx + p]) & 0x7FFFFFFFu);
         }
         s_mx[g][tid & (XM - 1)] = mx;
         const int col = n0 + (tid >> 3);
         mx = 0;
         if (col < n) {
-            const double *y = a.Y + (int64_t)col * a.ldy;
+            const double *y = a.Y + ES * (int64_t)col * a.ldy;
 #pragma unroll 8
-            for (int k = tid & 7; k < n; k += 8) mx = max(mx, (unsigned)__double2hiint(y[k]) & 0x7FFFFFFFu);
+            for (int k = tid & 7; k < ES * n; k += 8) mx = max(mx, (unsigned)__double2hiint(y[k]) & 0x7FFFFFFFu);
         }
 #pragma unroll
         for (int o = 4; o; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
@@ -235,33 +250,38 @@ xsplit_residual_kernel(XArgs a, const ResJob *__restrict__ jobs)
     const int row = m0 + 32 * qw + lane;
     if (warp == 0) {
         const bool go = n > kXsplitMinN && digits_accurate(s_ri, s_sj, min(XM, n - m0), min(XN, n - n0), lane,
-                                                           a.norm_a, (float)(cdiv_i(n, XM) * cdiv_i(n, XN)));
+                                                           a.norm_a, (float)(ES * cdiv_i(n, XM) * cdiv_i(n, XN)));
         if (lane == 0) s_go = go;
     }
     __syncthreads();
     if (!s_go) {
-        // FP64 products, in the order of residual_f64_kernel
+        // FP64 products, in the order of residual_f64_kernel and zresidual_f64_kernel
         double acc[16], ss = 0.0;
 #pragma unroll
         for (int j = 0; j < 16; ++j) acc[j] = 0.0;
         if (row < n) {
-            const double *x = a.X + row;
-            const double *y = a.Y + (int64_t)(n0 + 16 * cg) * a.ldy;
+            const double *x = a.X + ES * row;
+            const double *y = a.Y + ES * (int64_t)(n0 + 16 * cg) * a.ldy;
             const int jn = min(16, n - n0 - 16 * cg);
             if (jn > 0) {
 #pragma unroll 2
                 for (int k = 0; k < n; ++k) {
-                    const double xv = x[(int64_t)k * a.ldx];
+                    const double xv = x[ES * (int64_t)k * a.ldx];
+                    const double xi = CPLX ? (im ? 1.0 : -1.0) * x[ES * (int64_t)k * a.ldx + 1] : 0.0;
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) acc[j] = fma(xv, y[k + (int64_t)min(j, jn - 1) * a.ldy], acc[j]);
+                    for (int j = 0; j < 16; ++j) {
+                        const double *yj = y + ES * (k + (int64_t)min(j, jn - 1) * a.ldy);
+                        acc[j] = fma(xv, yj[im], acc[j]);
+                        if (CPLX) acc[j] = fma(xi, yj[1 - im], acc[j]);
+                    }
                 }
             }
 #pragma unroll
             for (int j = 0; j < 16; ++j) {
                 if (j >= jn) continue;
                 const int64_t col = n0 + 16 * cg + j;
-                const double r = (a.A[row + col * a.lda] - acc[j]) * a.sc;
-                a.Rhat[row + col * a.ldr] = (float)r;
+                const double r = (a.A[ES * (row + col * a.lda) + im] - acc[j]) * a.sc;
+                a.Rhat[ES * (row + col * a.ldr) + im] = (float)r;
                 ss = fma(r, r, ss);
             }
         }
@@ -292,30 +312,33 @@ xsplit_residual_kernel(XArgs a, const ResJob *__restrict__ jobs)
     long long hi[16], lo[16];
 #pragma unroll
     for (int j = 0; j < 16; ++j) hi[j] = lo[j] = 0;
-    const int KT = (n + XK - 1) / XK;
+    const int KS = (n + XK - 1) / XK, KT = ES * KS;  // steps of 64 terms, real parts first
     bool ok = true;
     int kt = 0;
     for (; kt < KT; ++kt) {
-        const int k0 = kt * XK, kc = min(XK, n - k0), ksteps = (kc + 15) / 16;
+        const int seg = CPLX && kt >= KS, k0 = (kt - seg * KS) * XK, kc = min(XK, n - k0), ksteps = (kc + 15) / 16;
         // digits of the rows of X and the columns of Y; rows and columns past
         // n are left as they are: they reach only outputs that are not stored
 #pragma unroll 1
         for (int u = tid; u < XM * (XK / 8); u += XT) {
             const int r = u & (XM - 1), c = u / XM;
             if (m0 + r >= n || c >= 2 * ksteps) continue;
-            const double *x = a.X + m0 + r + (int64_t)(k0 + 8 * c) * a.ldx;
+            const double *x = a.X + ES * (m0 + r + (int64_t)(k0 + 8 * c) * a.ldx) + seg;
             double v[8];
 #pragma unroll
-            for (int q = 0; q < 8; ++q) v[q] = 8 * c + q < kc ? x[(int64_t)q * a.ldx] : 0.0;
+            for (int q = 0; q < 8; ++q) {
+                v[q] = 8 * c + q < kc ? x[ES * (int64_t)q * a.ldx] : 0.0;
+                if (CPLX && seg && !im) v[q] = -v[q];
+            }
             store_digits(sA + r * 128 + ((c ^ (r & 7)) << 4), XA_BYTES, v, s_ri[r]);
         }
         {
             const int j = tid >> 3, c = tid & 7;
             if (n0 + j < n && c < 2 * ksteps) {
-                const double *y = a.Y + (int64_t)(n0 + j) * a.ldy + k0 + 8 * c;
+                const double *y = a.Y + ES * ((int64_t)(n0 + j) * a.ldy + k0 + 8 * c) + (seg ^ im);
                 double v[8];
 #pragma unroll
-                for (int q = 0; q < 8; ++q) v[q] = 8 * c + q < kc ? y[q] : 0.0;
+                for (int q = 0; q < 8; ++q) v[q] = 8 * c + q < kc ? y[ES * q] : 0.0;
                 store_digits(sB + j * 128 + ((c ^ (j & 7)) << 4), XB_BYTES, v, s_sj[j]);
             }
         }
@@ -373,10 +396,10 @@ xsplit_residual_kernel(XArgs a, const ResJob *__restrict__ jobs)
             const int c = 16 * cg + j, col = n0 + c;
             if (col >= n) continue;
             const int e = ri + s_sj[c];
-            double r = a.A[row + (int64_t)col * a.lda];
+            double r = a.A[ES * (row + (int64_t)col * a.lda) + im];
             r = sub_scaled(sub_scaled(r, hi[j], e - 36), lo[j], e - 68);
             const double rs = r * a.sc;
-            a.Rhat[row + (int64_t)col * a.ldr] = (float)rs;
+            a.Rhat[ES * (row + (int64_t)col * a.ldr) + im] = (float)rs;
             ss = fma(rs, rs, ss);
         }
     }
@@ -401,15 +424,31 @@ xsplit_residual_kernel(XArgs a, const ResJob *__restrict__ jobs)
 
 int xsplit_parts(int n) { return n <= 0 ? 0 : (int)(cdiv_i(n, XM) * cdiv_i(n, XN)); }
 
-cudaError_t launch_xsplit_residual(const double *A, int64_t lda, const double *X, int64_t ldx, int n, int e,
-                                   double norm_a, float *Rhat, int ldr, double *partials, int *nparts, cudaStream_t s)
+cudaError_t launch_xsplit_residual(const double *A, int64_t lda, const double *X, int64_t ldx, const double *Y,
+                                   int64_t ldy, int n, int shift, double norm_a, float *Rhat, int ldr, double *partials,
+                                   int *nparts, cudaStream_t s)
 {
     *nparts = xsplit_parts(n);
     if (n <= 0) return cudaSuccess;
-    cudaError_t err = allow_max_smem((const void *)xsplit_residual_kernel);
+    cudaError_t err = allow_max_smem((const void *)xsplit_residual_kernel<false>);
     if (err) return err;
-    xsplit_residual_kernel<<<dim3((unsigned)cdiv_i(n, XM), (unsigned)cdiv_i(n, XN)), XT, X_SMEM, s>>>(
-        XArgs{A, X, X, lda, ldx, ldx, Rhat, ldr, partials, ldexp(1.0, -2 * e), norm_a, n}, nullptr);
+    xsplit_residual_kernel<false><<<dim3((unsigned)cdiv_i(n, XM), (unsigned)cdiv_i(n, XN)), XT, X_SMEM, s>>>(
+        XArgs{A, X, Y, lda, ldx, ldy, Rhat, ldr, partials, ldexp(1.0, -shift), norm_a, n}, nullptr);
+    count_launch();
+    return cudaGetLastError();
+}
+
+cudaError_t launch_xsplit_zresidual(const double *A, int64_t lda, const double *X, int64_t ldx, int n, int shift,
+                                    double norm_a, cplx<float> *Rhat, int ldr, double *partials, int *nparts,
+                                    cudaStream_t s)
+{
+    *nparts = 2 * xsplit_parts(n);
+    if (n <= 0) return cudaSuccess;
+    cudaError_t err = allow_max_smem((const void *)xsplit_residual_kernel<true>);
+    if (err) return err;
+    xsplit_residual_kernel<true><<<dim3((unsigned)cdiv_i(n, XM), (unsigned)cdiv_i(n, XN), 2), XT, X_SMEM, s>>>(
+        XArgs{A, X, X, lda, ldx, ldx, reinterpret_cast<float *>(Rhat), ldr, partials, ldexp(1.0, -shift), norm_a, n},
+        nullptr);
     count_launch();
     return cudaGetLastError();
 }
@@ -417,9 +456,9 @@ cudaError_t launch_xsplit_residual(const double *A, int64_t lda, const double *X
 cudaError_t launch_xsplit_residual_batched(const ResJob *jobs, int batch, int nmax, cudaStream_t s)
 {
     if (nmax <= 0 || batch <= 0) return cudaSuccess;
-    cudaError_t err = allow_max_smem((const void *)xsplit_residual_kernel);
+    cudaError_t err = allow_max_smem((const void *)xsplit_residual_kernel<false>);
     if (err) return err;
-    xsplit_residual_kernel<<<dim3((unsigned)cdiv_i(nmax, XM), (unsigned)cdiv_i(nmax, XN), (unsigned)batch), XT, X_SMEM,
+    xsplit_residual_kernel<false><<<dim3((unsigned)cdiv_i(nmax, XM), (unsigned)cdiv_i(nmax, XN), (unsigned)batch), XT, X_SMEM,
                              s>>>(XArgs{}, jobs);
     count_launch();
     return cudaGetLastError();

@@ -94,3 +94,17 @@ def test_batch():
     assert torch.equal(X1[4], X2[4]) and torch.equal(X1[5], X2[5])  # n <= 32: FP64 products
     for x, y in zip(X1, X2):
         assert oracle.rel_err(x.cpu().numpy(), y.cpu().numpy()) <= 1e-13
+
+
+@pytest.mark.parametrize("n", [33, 64, 65, 129, 200])
+def test_complex_and_cube_root(n):
+    # two corrections from digit products and from FP64 products: both within
+    # rounding of the root
+    A = synth.shifted_gaussian(n, 3.0, seed=n)
+    for f, M in ((mp.sqrtm_mixed_complex, A + 1j * synth.shifted_gaussian(n, 0.0, seed=n + 1)), (mp.cbrtm_mixed, A)):
+        Md = torch.from_numpy(M).cuda()
+        X1, i1 = f(Md, steps=3)
+        X2, i2 = f(Md, steps=3, precision=mp.PREC_RESID_FP64)
+        assert i1["status"] == 0 and i2["status"] == 0
+        X1, X2 = X1.cpu().numpy(), X2.cpu().numpy()
+        assert np.linalg.norm(X1 - X2) <= 1e-13 * np.linalg.norm(X2)
