@@ -519,7 +519,7 @@ def run_ours(args):
                 "peak_one_sm": one_sm_peak, "frac_one_sm": achieved / one_sm_peak,
                 "note": f"peak derived ({sms} SMs x 128 FP32 lanes x 2 flop x {mhz:.0f} MHz, read from the "
                         "device), not measured; the "
-                        "bulge chain runs on one chase CTA (16 helper CTAs take the out-of-window "
+                        "bulge chain runs on one chase CTA (n/32 = 16 helper CTAs take the out-of-window "
                         "updates), so the one-SM fraction is the meaningful one; achieved and traffic "
                         "are per step, summed over the chase launches of one call (ncu dram bytes, "
                         "for this rqr.cu only)"}
