@@ -77,11 +77,12 @@ enum { SQRTM_KIND_AUTO = 0, SQRTM_KIND_GENERAL = 1, SQRTM_KIND_SPD = 2, SQRTM_KI
  * summed in FP64 (error-free splitting; the terms left out are below
  * n 2^(rho_i + rho_j - 56), 2^rho_i bounding row i of X, i.e. within the
  * FP64 product's own error bound).  The general path's residual (Algorithm
- * 2, step 4) of the FP32 method, alone or in a batch, real or complex, does
- * the same from n = 33 on, with the digit slices of the rows of X against
- * those of its columns; up to n = 1024 parts of the product where the digits
- * would be less accurate than FP64 (graded or far from normal X) are formed
- * in FP64.  RESID_FP64 forces the FP64 product on the CUDA cores in all. */
+ * 2, step 4) of the FP32 method, alone or in a batch, does the same from
+ * n = 33 on (complex iterates and one of the cube root's two products: up to
+ * n = 1024), with the digit slices of the rows of X against those of its
+ * columns; up to n = 1024 parts of the product where the digits would be less
+ * accurate than FP64 (graded or far from normal X) are formed in FP64.
+ * RESID_FP64 forces the FP64 product on the CUDA cores in all. */
 enum {
     SQRTM_PREC_AUTO = -1,
     SQRTM_PREC_FP32 = 0,
