@@ -385,9 +385,8 @@ qr_chase_kernel(const SchurDesc<R> *__restrict__ descs, int H)
     __shared__ cplx<R> s_prev[NB], s_defl[NB];  // the last multishift sweep's shifts; eigenvalues deflated since
     __shared__ R s_mnrm;
     __shared__ int s_prevn, s_prevhi, s_prefail;
-    __shared__ int s_lo, s_hi, s_iter, s_status, s_done, s_nb, s_sweeps, s_stop, s_nwin, s_nlog, s_small, s_bad, s_npost,
-        s_tiny;
-    __shared__ long long s_uoff, s_rots, s_work;
+    __shared__ int s_lo, s_hi, s_iter, s_status, s_done, s_nb, s_sweeps, s_stop, s_small, s_bad, s_tiny;
+    __shared__ long long s_rots, s_work;
 
     const SchurDesc<R> d = descs[HELP ? 0 : blockIdx.x];
     if (HELP && blockIdx.x > 0) {
@@ -414,20 +413,23 @@ qr_chase_kernel(const SchurDesc<R> *__restrict__ descs, int H)
         s_iter = st[1];
         s_status = 0;
         s_done = 0;
-        s_nlog = 0;
-        s_nwin = 0;
-        s_uoff = 0;
         s_sweeps = st[4];
         s_rots = (long long)st[5] + ((long long)st[6] << 31);
         s_work = (long long)st[8] + ((long long)st[9] << 31);
         s_stop = 0;
         s_bad = 0;
-        s_npost = 0;
         s_prevn = 0;
         s_prevhi = 0;
     }
     __syncthreads();
 
+    // log, window, U and posted-window counts: the same in every thread.  (In
+    // shared memory, advanced by thread 0 at the end of a window, a window that
+    // covers its whole active block had no barrier between a late warp's use of
+    // the log position and the advance: its rotations went to the next
+    // window's place.)
+    int nlog = 0, nwin = 0, npost = 0;
+    long long uoff = 0;
     while (true) {
         const int hi = s_hi;
         if (hi <= 0) { if (tid == 0) s_done = 1; break; }
@@ -455,12 +457,12 @@ qr_chase_kernel(const SchurDesc<R> *__restrict__ descs, int H)
             int nb = min(NB, max(1, (m - 2) / 4));
             s_tiny = m <= kQrTiny;
             const long long nwin_sweep = s_tiny ? 1 : ((hi - lo) + 3 * (nb - 1) + W - 1) / W;
-            const bool fits = s_nlog + nwin_sweep * (W * NB) <= d.log_cap && s_nwin + nwin_sweep <= d.win_cap &&
-                              s_uoff + nwin_sweep * (long long)(D::RR * D::RR) <= d.u_cap;
+            const bool fits = nlog + nwin_sweep * (W * NB) <= d.log_cap && nwin + nwin_sweep <= d.win_cap &&
+                              uoff + nwin_sweep * (long long)(D::RR * D::RR) <= d.u_cap;
             s_small = 0;
             if (!fits) {
                 s_stop = 1;  // drain the log first
-                if (s_nlog == 0 && s_nwin == 0 && s_uoff == 0) s_status = 7;  // can never fit
+                if (nlog == 0 && nwin == 0 && uoff == 0) s_status = 7;  // can never fit
             } else {
                 if (lo > 0) T[lo + (int64_t)(lo - 1) * ld] = cplx<R>{0, 0};
             }
@@ -500,19 +502,19 @@ qr_chase_kernel(const SchurDesc<R> *__restrict__ descs, int H)
             // the sweep that split it off)
             const int m = hi - lo + 1;
             const int nc = s_prevn;
-            if (tid < nc) d.log[s_nlog + tid] = RotLog<R>{R(0), s_prev[tid].x, s_prev[tid].y, R(0)};
+            if (tid < nc) d.log[nlog + tid] = RotLog<R>{R(0), s_prev[tid].x, s_prev[tid].y, R(0)};
             if (tid == 0) {
                 WinRec wr;
-                wr.start = s_nlog; wr.kbase = lo; wr.nsteps = -1; wr.kmin = lo; wr.rr = m;
+                wr.start = nlog; wr.kbase = lo; wr.nsteps = -1; wr.kmin = lo; wr.rr = m;
                 wr.lo = lo; wr.hi = hi; wr.t0 = 0; wr.nb = nc; wr.r0 = lo; wr.rnext = hi; wr.pad = 1;
-                wr.uoff = s_uoff;
-                d.win[s_nwin] = wr;
-                s_nwin += 1;
-                s_uoff += (long long)m * m;
-                s_nlog += NB;
+                wr.uoff = uoff;
+                d.win[nwin] = wr;
                 s_hi = lo - 1;
                 s_iter = 0;
             }
+            nwin += 1;
+            uoff += (long long)m * m;
+            nlog += NB;
             __syncthreads();
             continue;
         }
@@ -628,6 +630,7 @@ qr_chase_kernel(const SchurDesc<R> *__restrict__ descs, int H)
                             q[i] = cplx<R>{0, 0};
                         }
                     }
+                    __syncwarp();  // every lane's loads before any lane's stores
                     if (act && k == lo) x = x - s_mu[g];
                     R c = R(1);
                     cplx<R> s{0, 0}, r{0, 0};
@@ -676,24 +679,24 @@ qr_chase_kernel(const SchurDesc<R> *__restrict__ descs, int H)
                     for (int b = warp; b < bw; b += NCH / 32)
                         for (int a = lane; a <= min(b + 2, bw - 1); a += 32)
                             T[(r0 + a) + (int64_t)(r0 + b) * ld] = blk[a + b * BLD];
-                    RotLog<R> *dst = d.log + s_nlog;
+                    RotLog<R> *dst = d.log + nlog;
                     for (int e = tid; e < W * NB; e += NCH) dst[e] = rt[e];
                     if (tid == 0) {
                         WinRec wr;
-                        wr.start = s_nlog; wr.kbase = kbase; wr.nsteps = ns; wr.kmin = kmin; wr.rr = rr;
+                        wr.start = nlog; wr.kbase = kbase; wr.nsteps = ns; wr.kmin = kmin; wr.rr = rr;
                         wr.lo = lo; wr.hi = hi; wr.t0 = t0; wr.nb = nb; wr.r0 = r0; wr.rnext = rnext; wr.pad = 0;
-                        wr.uoff = s_uoff;
-                        d.win[s_nwin] = wr;
-                        d.postlist[s_npost] = s_nwin;
+                        wr.uoff = uoff;
+                        d.win[nwin] = wr;
+                        d.postlist[npost] = nwin;
                     }
                     __threadfence();
                     chase_bar<NCH>();
-                    if (tid == 0) atomicExch(&d.sync[0], s_npost + 1);
+                    if (tid == 0) atomicExch(&d.sync[0], npost + 1);
                 }
             } else if (pre_cn > 0) {
                 constexpr int NPRE = kQrThreads - NB * 16;  // threads of the warps that do not chase
                 static_assert(NPRE >= 32, "the prefetch needs a warp");
-                if (warp == NB / 2 && !warp_poll_helpers(d, H, s_npost) && lane == 0) s_prefail = 1;
+                if (warp == NB / 2 && !warp_poll_helpers(d, H, npost) && lane == 0) s_prefail = 1;
                 asm volatile("bar.sync 2, %0;" ::"n"(NPRE) : "memory");
                 if (!s_prefail) {
                     const int pt = tid - NB * 16;
@@ -714,25 +717,25 @@ qr_chase_kernel(const SchurDesc<R> *__restrict__ descs, int H)
                 for (int b = warp; b < bw; b += nt / 32)
                     for (int a = lane; a <= min(b + 2, bw - 1); a += 32)
                         T[(r0 + a) + (int64_t)(r0 + b) * ld] = blk[a + b * BLD];
-                RotLog<R> *dst = d.log + s_nlog;
+                RotLog<R> *dst = d.log + nlog;
                 for (int e = tid; e < W * NB; e += nt) dst[e] = rt[e];
             }
             if (HELP && pre_cn == 0) {
                 if (post && tid == 0) {
                     WinRec wr;
-                    wr.start = s_nlog; wr.kbase = kbase; wr.nsteps = ns; wr.kmin = kmin; wr.rr = rr;
+                    wr.start = nlog; wr.kbase = kbase; wr.nsteps = ns; wr.kmin = kmin; wr.rr = rr;
                     wr.lo = lo; wr.hi = hi; wr.t0 = t0; wr.nb = nb; wr.r0 = r0; wr.rnext = rnext; wr.pad = 0;
-                    wr.uoff = s_uoff;
-                    d.win[s_nwin] = wr;
-                    d.postlist[s_npost] = s_nwin;
+                    wr.uoff = uoff;
+                    d.win[nwin] = wr;
+                    d.postlist[npost] = nwin;
                 }
                 __threadfence();
                 __syncthreads();
-                if (post && tid == 0) atomicExch(&d.sync[0], s_npost + 1);
+                if (post && tid == 0) atomicExch(&d.sync[0], npost + 1);
                 // helpers done with every window posted before this one (all of
                 // them if this one is done here; for a posted one the warps that
                 // prefetched its new columns have waited for that already)
-                if (!wait_helpers(d, H, s_npost)) {
+                if (!wait_helpers(d, H, npost)) {
                     if (tid == 0) s_status = 6;
                     __syncthreads();
                     break;
@@ -786,26 +789,26 @@ qr_chase_kernel(const SchurDesc<R> *__restrict__ descs, int H)
                 __syncthreads();
             }
             if (tid == 0) {
-                if (post) ++s_npost;
                 if (!post) {
                     WinRec wr;
-                    wr.start = s_nlog; wr.kbase = kbase; wr.nsteps = ns; wr.kmin = kmin; wr.rr = rr;
+                    wr.start = nlog; wr.kbase = kbase; wr.nsteps = ns; wr.kmin = kmin; wr.rr = rr;
                     wr.lo = lo; wr.hi = hi; wr.t0 = t0; wr.nb = nb; wr.r0 = r0; wr.rnext = rnext; wr.pad = 0;
-                    wr.uoff = s_uoff;
-                    d.win[s_nwin] = wr;
+                    wr.uoff = uoff;
+                    d.win[nwin] = wr;
                 }
-                s_nwin += 1;
-                s_uoff += (long long)rr * rr;
-                s_nlog += W * NB;
                 if (s_bad) s_status = 7;
             }
+            if (post) ++npost;
+            nwin += 1;
+            uoff += (long long)rr * rr;
+            nlog += W * NB;
             if (HELP) __threadfence();  // the block and head columns, before the next block is read back
             __syncthreads();
         }
         __syncthreads();
         // cooperative chase: the whole sweep's out-of-window updates are done
         // before the next sweep reads T
-        if (HELP && !s_status && !wait_helpers(d, H, s_npost)) {
+        if (HELP && !s_status && !wait_helpers(d, H, npost)) {
             if (tid == 0) s_status = 6;
             __syncthreads();
         }
@@ -816,9 +819,9 @@ qr_chase_kernel(const SchurDesc<R> *__restrict__ descs, int H)
         st[0] = s_hi;
         st[1] = s_iter;
         st[2] = (s_done || s_status) ? 1 : 0;
-        st[3] = s_nlog;
-        st[7] = s_nwin;
-        d.rstate[0] = s_nwin;
+        st[3] = nlog;
+        st[7] = nwin;
+        d.rstate[0] = nwin;
         st[4] = s_sweeps;
         st[5] = (int)(s_rots & 0x7fffffff);
         st[6] = (int)(s_rots >> 31);
