@@ -50,7 +50,9 @@ SQRTM_API int sqrtm_step_hessenberg(sqrtm_handle_t h, const double *dA, int64_t 
 
 /* Complex Schur decomposition (Algorithm 2, step 1): dT (in: A_s, out: T
  * upper triangular) and dQ (out: unitary) with A_s = Q T Q^H: Householder
- * Hessenberg reduction, then single-shift QR sweeps.  Returns 0 or 3. */
+ * Hessenberg reduction, then the QR iteration that the solver takes for such
+ * an A_s: in FP32 (fp64 = 0), where no entry has an imaginary part, double-
+ * shift sweeps in real arithmetic, else single-shift ones.  Returns 0 or 3. */
 SQRTM_API int sqrtm_step_schur(sqrtm_handle_t h, void *dT, void *dQ, int64_t n, int fp64);
 
 /* Symmetric eigendecomposition (Algorithm 3, step 1) of the real symmetric

@@ -64,37 +64,78 @@ extern "C" int sqrtm_step_scale(sqrtm_handle_t h, const double *dA, int64_t n, i
 }
 
 template <class R>
+__global__ void any_imag_kernel(const cplx<R> *__restrict__ T, int64_t count, int *flag)
+{
+    bool any = false;
+    for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < count; t += (int64_t)gridDim.x * blockDim.x)
+        any = any || !(T[t].y == R(0));
+    if (__syncthreads_or(any) && threadIdx.x == 0) *flag = 1;
+}
+
+// The QR iteration is the solver's own for such an A_s: in FP32 the real one
+// where no entry has an imaginary part (with the solver's two buffer sets,
+// helpers and deferred passes on the side stream), else the complex one with
+// one CTA.
+template <class R>
 static int schur_step(sqrtm_handle_t h, cplx<R> *T, cplx<R> *Q, int64_t n)
 {
     StepScratch ss; void *ex;
-    size_t extra = Carve::round((n + 8) * sizeof(cplx<R>)) + Carve::round(8 * sizeof(R)) + Carve::round(sizeof(SchurDesc<R>)) +
-                   Carve::round(qr_log_capacity(n) * sizeof(RotLog<R>)) + Carve::round(kQrStateInts * sizeof(int)) +
-                   Carve::round(4 * sizeof(int)) +
-                   Carve::round(qr_win_capacity(n) * sizeof(WinRec)) + Carve::round(qr_u_capacity(n) * sizeof(cplx<R>));
+    const size_t nn = (size_t)n * n;
+    const bool maybe_real = sizeof(R) == sizeof(float);
+    const int sets = maybe_real ? 2 : 1;
+    size_t extra = Carve::round((n + 8) * sizeof(cplx<R>)) + Carve::round(8 * sizeof(R)) +
+                   Carve::round(2 * sizeof(SchurDesc<R>)) + Carve::round(kQrStateInts * sizeof(int)) +
+                   Carve::round(4 * sizeof(int)) + Carve::round(kQrSyncInts * sizeof(int)) +
+                   Carve::round(qr_win_capacity(n) * sizeof(int)) + (maybe_real ? Carve::round(nn * sizeof(cplx<R>)) : 0) +
+                   sets * (Carve::round(qr_log_capacity(n) * sizeof(RotLog<R>)) +
+                           Carve::round(qr_win_capacity(n) * sizeof(WinRec)) +
+                           Carve::round(qr_u_capacity(n) * sizeof(cplx<R>)));
     if (int rc = step_scratch(h, n, extra, &ss, &ex)) return rc;
     Carve c(ex);
     cplx<R> *v = c.take<cplx<R>>(n + 8);
     R *beta = c.take<R>(8);
-    SchurDesc<R> *dd = c.take<SchurDesc<R>>(1);
-    RotLog<R> *rlog = c.take<RotLog<R>>(qr_log_capacity(n));
+    SchurDesc<R> *dd = c.take<SchurDesc<R>>(2);
     int *qstate = c.take<int>(kQrStateInts);
-    WinRec *wrec = c.take<WinRec>(qr_win_capacity(n));
-    cplx<R> *ubuf = c.take<cplx<R>>(qr_u_capacity(n));
     int *rstate = c.take<int>(4);
-    SchurDesc<R> hd;
-    hd.rstate = rstate;
-    hd.sync = nullptr;
-    hd.postlist = nullptr;
-    hd.T = T; hd.Q = Q; hd.v = v; hd.beta = beta; hd.status = ss.iscal + 1; hd.n = (int)n; hd.ld = (int)n;
-    hd.counters = nullptr;
-    hd.log = rlog; hd.state = qstate; hd.log_cap = (int)std::min<int64_t>(qr_log_capacity(n), INT32_MAX);
-    hd.win = wrec; hd.win_cap = (int)std::min<int64_t>(qr_win_capacity(n), INT32_MAX);
-    hd.ubuf = ubuf; hd.u_cap = qr_u_capacity(n);
-    memcpy(h->staging.p, &hd, sizeof(hd));
+    int *qsync = c.take<int>(kQrSyncInts);
+    int *qpost = c.take<int>(qr_win_capacity(n));
+    bool real = false;
+    if (maybe_real) {
+        any_imag_kernel<R><<<(int)std::min<int64_t>(592, cdiv_i((int64_t)nn, 256)), 256, 0, h->stream>>>(T, (int64_t)nn, ss.iscal + 2);
+        count_launch();
+        int any = 0;
+        if (cudaGetLastError() || fetch(h, &any, ss.iscal + 2, sizeof(int))) return 7;
+        real = any == 0;
+    }
+    SchurDesc<R> hd[2];
+    for (int q = 0; q < 2; ++q) {
+        SchurDesc<R> &d = hd[q];
+        if (q >= sets) { d = hd[0]; break; }
+        d.rstate = rstate + 2 * q;
+        d.sync = real ? qsync : nullptr;
+        d.postlist = real ? qpost : nullptr;
+        d.T = T; d.Q = Q; d.v = v; d.beta = beta; d.status = ss.iscal + 1; d.n = (int)n; d.ld = (int)n;
+        d.counters = nullptr;
+        d.state = qstate; d.log_cap = (int)std::min<int64_t>(qr_log_capacity(n), INT32_MAX);
+        d.log = c.take<RotLog<R>>(qr_log_capacity(n));
+        d.win = c.take<WinRec>(qr_win_capacity(n));
+        d.win_cap = (int)std::min<int64_t>(qr_win_capacity(n), real ? std::max<int64_t>(64, n / 2) : INT32_MAX);
+        d.ubuf = c.take<cplx<R>>(qr_u_capacity(n)); d.u_cap = qr_u_capacity(n);
+        d.wait_ns = h->wait_ns;
+    }
+    if (maybe_real) hd[0].w = hd[1].w = c.take<cplx<R>>(nn);
+    memcpy(h->staging.p, hd, sizeof(hd));
     if (cudaMemcpyAsync(dd, h->staging.p, sizeof(hd), cudaMemcpyHostToDevice, h->stream)) return 7;
     if (cudaStreamSynchronize(h->stream)) return 7;
     if (launch_hessenberg<R>(dd, 1, (int)n, 64, h->stream)) return 7;
-    if (launch_qr_sweeps<R>(dd, 1, (int)n, (int *)h->staging.p + 512, qstate, h->stream)) return 7;
+    int *hstate = (int *)h->staging.p + 512;
+    if constexpr (sizeof(R) == sizeof(float)) {
+        const sqrtm_tune_entry *tune = tune_for(h, n);
+        if (real && launch_rqr_sweeps(dd, (int)n, hstate, qstate, h->stream, nullptr, dd + 1, h->side, h->qev, qsync,
+                                      tune ? tune->qr_helpers : -1))
+            return 7;
+    }
+    if (!real && launch_qr_sweeps<R>(dd, 1, (int)n, hstate, qstate, h->stream)) return 7;
     int st = 0;
     if (fetch(h, &st, ss.iscal + 1, sizeof(int))) return 7;
     return st;
