@@ -68,7 +68,10 @@ constexpr int kStep = 352;           // threads that take part in a step (11 war
 constexpr int kQuad = 128;           // threads of a group that applies a window to 32 segments
 constexpr int KB = 4;                // steps between two barriers of such a group
 constexpr int NAH = 11;              // column triples ahead of the chain
-constexpr int kShiftIt = 10;         // iterations of the shift refinement
+constexpr int kShiftIt = 12;         // iterations of the shift refinement (of a large active block)
+constexpr float kShiftTol = 3e-2f;   // and its tolerance relative to the spread of the estimates
+constexpr int kShiftSlow = 6;        // after this many sweeps without deflation the refinement starts anew
+constexpr int kShiftItSlow = 30;     // and may take this many iterations
 constexpr int kRqrPostMin = 64;      // fewer out-of-window rows + columns: the chase CTA does them
 constexpr int SLD = 81;              // staged segments: leading dimension (odd, >= RR)
 constexpr int kStage = kCta / kQuad * 32 * SLD;  // staged floats: 32 segments per group of four warps
@@ -223,15 +226,15 @@ __device__ __forceinline__ void tile_update(float a[3][3], Refl l, Refl r)
         }
     }
 }
-// First reflector of a bulge with shifts alpha +- sqrt(-q): from the first
-// column of (H - s1)(H - s2) for the block starting at lo.  B(i, j) is
-// element (i, j) at B[i + j ld].
-__device__ __noinline__ Refl intro_reflector(const float *B, int ld, int lo, float alpha, float q)
+// First reflector of a bulge with shifts alpha +- i r (r >= 0) or alpha +- r
+// (r < 0): from the first column of (H - s1)(H - s2) for the block starting at
+// lo.  B(i, j) is element (i, j) at B[i + j ld].
+__device__ __noinline__ Refl intro_reflector(const float *B, int ld, int lo, float alpha, float r)
 {
     const float a = B[lo + lo * ld], b = B[lo + (lo + 1) * ld], c = B[(lo + 1) + lo * ld],
                 d = B[(lo + 1) + (lo + 1) * ld], e = B[(lo + 2) + (lo + 1) * ld];
     const float am = a - alpha, dm = d - alpha;
-    float x0 = fmaf(am, am, fmaf(b, c, q)), x1 = c * (am + dm), x2 = c * e;
+    float x0 = fmaf(am, am, fmaf(b, c, r * fabsf(r))), x1 = c * (am + dm), x2 = c * e;
     const float m = fmaxf(fabsf(x0), fmaxf(fabsf(x1), fabsf(x2)));
     Refl v{0.0f, 0.0f, 0.0f};
     if (m > 0.0f) {
@@ -597,13 +600,20 @@ __device__ __noinline__ bool quad_window(float *vec, int stride, bool on, const 
 // 32, leading dimension MLD) refined together by the Ehrlich-Aberth
 // iteration with Hyman's recurrence (the method of cta_aberth_shifts in
 // qr_small.cuh, here for real M: the running sums take two multiply-adds per
-// entry instead of four).  On entry z holds m distinct estimates; true: the
-// last corrections were at most tol (|z| + 1e-3 max|M|).  Shifts need not be
-// eigenvalues to rounding: the correction that passes the test is itself
-// applied, and the iteration converges cubically (tol 1e-2 and at most
-// kShiftIt iterations against 1e-4 and 24: 0.5 times the iterations, the same
-// number of steps within their spread).  Every thread of the CTA calls it.
-
+// entry instead of four).  M is the trailing block as centre_block leaves it,
+// mnrm its largest entry.  The QR iteration does not see a translation, so
+// every tolerance here and in the two functions below is relative to the
+// spread of the estimates, max|z|, and not to the eigenvalues' distance from
+// zero: relative to that, matrices as near to a multiple of I as 300 I + G /
+// sqrt(n) ran into the iteration cap.  (Nor is it relative to mnrm, which in a
+// graded M lies far above the eigenvalues: with 10^(10 (j - i) / n) on the
+// entries they ran into it as well.)  On entry z holds m distinct estimates;
+// true: the last corrections were at most kShiftTol max|z|.  Shifts need not
+// be eigenvalues to rounding: the correction that passes the test is itself
+// applied, and the iteration converges cubically.  An iteration costs about ten
+// steps of a sweep, so at most 6 + (rows of the active block) / 32 of them, up
+// to kShiftIt, are taken: ms of chase with 10 / 14 at n = 64 0.452 / 0.462, 200
+// 2.28 / 2.36, 512 9.93 / 9.86, 2048 105.2 / 106.3.
 //
 // A half-warp per estimate (warps 0 .. 15 take 32), lane r of it keeping the
 // sums of rows r and r + 16, as packed pairs (re, im): the packed FP32
@@ -642,6 +652,11 @@ __device__ __forceinline__ f2 f2_add(f2 a, f2 b)
     asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
     return r;
 }
+// largest of a warp's non-negative values
+__device__ __forceinline__ float warp_max(float v)
+{
+    return __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(v)));
+}
 // 1 / (x + i y) to about 1e-6 (an estimate of an estimate: shifts only);
 // a zero or overflowing modulus gives zero
 __device__ __forceinline__ float2 crcp_approx(float x, float y)
@@ -664,7 +679,6 @@ __device__ __noinline__ bool cta_aberth_real(const float *M, int m, float2 *z, f
     __builtin_assume(__isShared(M));
     __builtin_assume(__isShared(z));
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const float tol = 1e-2f;
     const float floor_sub = mnrm * 1e-20f;
     if (tid < m) {
         float sb = tid ? M[tid + (tid - 1) * MLD] : 1.0f;
@@ -745,12 +759,15 @@ __device__ __noinline__ bool cta_aberth_real(const float *M, int m, float2 *z, f
         }
         __syncthreads();
         bool done = true;
-        if (tid < m) {
-            const float2 w = s_w[tid];
-            const float2 zn = make_float2(z[tid].x - w.x, z[tid].y - w.y);
-            if (!(isfinite(zn.x) && isfinite(zn.y))) s_bad = 1;
-            done = fmaxf(fabsf(w.x), fabsf(w.y)) <= tol * (fmaxf(fabsf(zn.x), fabsf(zn.y)) + 1e-3f * mnrm);
-            z[tid] = zn;
+        if (warp == 0) {  // (m <= 32)
+            const float2 w = lane < m ? s_w[lane] : make_float2(0.0f, 0.0f);
+            float2 zn = make_float2(0.0f, 0.0f);
+            if (lane < m) {
+                zn = make_float2(z[lane].x - w.x, z[lane].y - w.y);
+                if (!(isfinite(zn.x) && isfinite(zn.y))) s_bad = 1;
+                z[lane] = zn;
+            }
+            done = fmaxf(fabsf(w.x), fabsf(w.y)) <= kShiftTol * warp_max(fmaxf(fabsf(zn.x), fabsf(zn.y)));
         }
         const int all = __syncthreads_and(done);
         if (s_bad) return false;
@@ -759,19 +776,48 @@ __device__ __noinline__ bool cta_aberth_real(const float *M, int m, float2 *z, f
     return false;
 }
 
-// Starting estimates (one warp; lane q holds the q-th previous estimate).
+// M (m x m) less the mean of its diagonal, times a power of two that takes its
+// largest entry to [1, 2).  Every thread of the CTA calls it, behind a barrier;
+// mnrm (shared) is 0 on entry.  Returns the mean, that power's inverse and
+// the largest entry.
+__device__ __noinline__ float3 centre_block(float *M, int m, float *mnrm)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = kCta / 32;
+    const float ctr = warp_sum(lane < m ? M[lane + lane * MLD] : 0.0f) * rcp_approx((float)m);
+    float mx = 0.0f;
+#pragma unroll 1
+    for (int j = warp; j < m; j += nw)
+        if (lane < m) mx = fmaxf(mx, fabsf(M[lane + j * MLD] - (lane == j ? ctr : 0.0f)));
+    mx = warp_max(mx);
+    if (lane == 0) atomicMax(reinterpret_cast<int *>(mnrm), __float_as_int(mx));  // (non-negative: ordered as integers)
+    __syncthreads();
+    mx = *mnrm;
+    const unsigned ex = min(max(__float_as_uint(mx) >> 23, 1u), 253u);
+    const float sc = __uint_as_float((254u - ex) << 23);
+#pragma unroll 1
+    for (int j = warp; j < m; j += nw)
+        if (lane < m) M[lane + j * MLD] = (M[lane + j * MLD] - (lane == j ? ctr : 0.0f)) * sc;
+    __syncthreads();
+    return make_float3(ctr, __uint_as_float(ex << 23), mx * sc);
+}
+
+// Starting estimates (one warp; lane q holds the q-th previous estimate).  prev
+// and defl are eigenvalues of the matrix, ctr the mean that centre_block took
+// from M, 1 / isc its scale.
 // Warm start: the np estimates of the previous sweep, whose trailing block
 // ended dh rows lower; for each of the dh eigenvalues deflated since (defl)
 // the nearest is dropped, and at most m stay; the remaining places (all for a
 // cold start, np = 0) take eigenvalues of M's 2 x 2 diagonal blocks.
-__device__ __noinline__ void warp_shift_start(const float *M, int m, float mnrm, const float2 *prev, int np, const float2 *defl,
-                                 int dh, float2 *z)
+__device__ __noinline__ void warp_shift_start(const float *M, int m, float mnrm, float ctr, float isc, const float2 *prev, int np,
+                                              const float2 *defl, int dh, float2 *z)
 {
     const int lane = threadIdx.x & 31;
-    const float2 c = lane < np ? prev[lane] : make_float2(0.0f, 0.0f);
+    float2 c = lane < np ? prev[lane] : make_float2(0.0f, 0.0f);
+    const float sc = rcp_approx(isc);  // (a power of two)
+    c = make_float2((c.x - ctr) * sc, c.y * sc);
     bool alive = lane < np;
     for (int q = 0; q < dh; ++q) {
-        const float ex = c.x - defl[q].x, ey = c.y - defl[q].y;
+        const float ex = c.x - (defl[q].x - ctr) * sc, ey = c.y - defl[q].y * sc;
         // the distance's leading bits with the lane below them
         const unsigned key = alive ? (__float_as_uint(fmaf(ex, ex, ey * ey)) & ~31u) | lane : 0xffffffffu;
         const unsigned best = __reduce_min_sync(0xffffffffu, key);
@@ -784,6 +830,14 @@ __device__ __noinline__ void warp_shift_start(const float *M, int m, float mnrm,
     const int cnt = __popc(__ballot_sync(0xffffffffu, alive));
     const unsigned am = __ballot_sync(0xffffffffu, alive);
     if (alive) z[__popc(am & ((1u << lane) - 1u))] = c;
+    // the spread as the 2 x 2 blocks show it (a diagonal scaling of M does not
+    // change it, where the largest entry of a graded M says nothing)
+    float spread = 0.0f;
+    if (lane < m) {
+        spread = fabsf(M[lane + lane * MLD]);
+        if (lane + 1 < m) spread = fmaxf(spread, sqrtf(fabsf(M[lane + (lane + 1) * MLD] * M[(lane + 1) + lane * MLD])));
+    }
+    spread = 5e-2f * fmaxf(warp_max(spread), 1e-6f * mnrm);
     const int q = lane - cnt;  // places cnt .. m-1
     if (q >= 0 && lane < m) {
         // an eigenvalue of the 2 x 2 diagonal block (q & ~1, q | 1), the
@@ -794,23 +848,23 @@ __device__ __noinline__ void warp_shift_start(const float *M, int m, float mnrm,
         const float r = ((q & 1) ? -1.0f : 1.0f) * sqrtf(fabsf(disc)), mid = 0.5f * (a + d);
         float sn, cs;
         sincospif((2.0f * q + 0.5f) / (float)m, &sn, &cs);
-        sn *= 1e-2f * mnrm;
-        cs *= 1e-2f * mnrm;
+        sn *= spread;
+        cs *= spread;
         z[lane] = disc < 0.0f ? make_float2(mid + cs, r + sn) : make_float2(mid + r + cs, sn);
     }
     __syncwarp();
 }
 
-// The m estimates z as bulges: sh[g] = (alpha, q) with shifts alpha +-
-// sqrt(-q): a conjugate pair alpha +- i beta gives q = beta^2, two real
-// estimates q = -((a - b) / 2)^2.  One warp; returns the number of bulges
-// (at most nb, at least 1).
-__device__ __noinline__ int warp_pair_shifts(const float2 *z, int m, float mnrm, float2 *sh, int nb)
+// The m estimates z (of M, see above) as bulges: sh[g] = (alpha, r) for
+// intro_reflector, in the matrix's own scale (isc = 1 / sc): a conjugate pair
+// alpha +- i beta gives r = beta, two real estimates r = -|a - b| / 2.  One
+// warp; returns the number of bulges (at most nb, at least 1).
+__device__ __noinline__ int warp_pair_shifts(const float2 *z, int m, float ctr, float isc, float2 *sh, int nb)
 {
     const int lane = threadIdx.x & 31;
     const float2 c = lane < m ? z[lane] : make_float2(0.0f, 0.0f);
-    const float thr = 1e-3f * (hypotf(c.x, c.y) + 1e-3f * mnrm);
     const bool in = lane < m;
+    const float thr = 1e-3f * warp_max(fmaxf(fabsf(c.x), fabsf(c.y)));
     unsigned up = __ballot_sync(0xffffffffu, in && c.y > thr);
     const unsigned dn = __ballot_sync(0xffffffffu, in && c.y < -thr);
     const unsigned re = __ballot_sync(0xffffffffu, in && fabsf(c.y) <= thr);
@@ -820,7 +874,7 @@ __device__ __noinline__ int warp_pair_shifts(const float2 *z, int m, float mnrm,
     const unsigned lt = (1u << lane) - 1u;
     if ((up >> lane) & 1u) {
         const int k = __popc(up & lt);
-        if (k < nb) sh[k] = make_float2(c.x, c.y * c.y);
+        if (k < nb) sh[k] = make_float2(fmaf(c.x, isc, ctr), fabsf(c.y) * isc);
     }
     // the r-th real estimate pairs with the (r ^ 1)-th
     __shared__ float s_re[32];
@@ -831,8 +885,7 @@ __device__ __noinline__ int warp_pair_shifts(const float2 *z, int m, float mnrm,
     const float other = isr && (rk ^ 1) < nr ? s_re[rk ^ 1] : c.x;
     if (isr && !(rk & 1)) {
         const int k = nu + (rk >> 1);
-        const float h = 0.5f * (c.x - other);
-        if (k < nb) sh[k] = make_float2(0.5f * (c.x + other), -h * h);
+        if (k < nb) sh[k] = make_float2(fmaf(0.5f * (c.x + other), isc, ctr), -0.5f * fabsf(c.x - other) * isc);
     }
     __syncwarp();
     return max(1, min(nb, nu + (nr + 1) / 2));
@@ -1043,7 +1096,7 @@ rqr_chase_kernel(const SchurDesc<float> *__restrict__ descs, int H, int nlo, int
     extern __shared__ __align__(16) unsigned char smraw[];
     float *tab = reinterpret_cast<float *>(smraw);        // two tables of W rows, used in turn
     float *dyn = tab + 2 * W * TS;
-    __shared__ float2 s_sh[NB];                           // the sweep's shifts (alpha, q)
+    __shared__ float2 s_sh[NB];                           // the sweep's shifts (alpha, r)
     __shared__ float s_m[NS2 * MLD];
     __shared__ float2 s_z[NS2], s_prev[NS2], s_defl[NS2];
     __shared__ int s_pair[128], s_cnt[4];
@@ -1167,7 +1220,8 @@ rqr_chase_kernel(const SchurDesc<float> *__restrict__ descs, int H, int nlo, int
             copy_cols(ms, ms, warp, nt / 32, [&](int i, int j) { return i <= j + 1 ? at(b0 + i, b0 + j) : 0.0f; },
                       [&](int i, int j, float v) { s_m[i + j * MLD] = v; });
             const int dh = s_prevhi - hi;
-            const bool warm = s_prevn > 0 && dh >= 0 && dh < ms;
+            const bool slow = s_iter > kShiftSlow;
+            const bool warm = s_prevn > 0 && dh >= 0 && dh < ms && !slow;
             if (warm && tid < dh) {
                 // an eigenvalue estimate of each deflated row: its diagonal
                 // entry, or the pair of the 2 x 2 block it heads or ends
@@ -1184,25 +1238,21 @@ rqr_chase_kernel(const SchurDesc<float> *__restrict__ descs, int H, int nlo, int
                 s_defl[tid] = make_float2(re, im);
             }
             __syncthreads();
-            {  // max |M_ij| (non-negative floats compare as integers)
-                float mx = 0.0f;
-                for (int j = warp; j < ms; j += nt / 32) mx = fmaxf(mx, lane < ms ? fabsf(s_m[lane + j * MLD]) : 0.0f);
-                const unsigned u = __reduce_max_sync(0xffffffffu, __float_as_uint(mx));
-                if (lane == 0) atomicMax(reinterpret_cast<int *>(&s_mnrm), (int)u);
-            }
+            const float3 cb = centre_block(s_m, ms, &s_mnrm);
+            const float ctr = cb.x, isc = cb.y, mnrm = cb.z;
+            if (warp == 0)
+                warp_shift_start(s_m, ms, mnrm, ctr, isc, s_prev, warm ? s_prevn : 0, s_defl, warm ? dh : 0, s_z);
             __syncthreads();
-            if (warp == 0) warp_shift_start(s_m, ms, s_mnrm, s_prev, warm ? s_prevn : 0, s_defl, warm ? dh : 0, s_z);
-            __syncthreads();
-            cta_aberth_real(s_m, ms, s_z, s_mnrm, kShiftIt);
-            // (unconverged estimates are shifts all the same; non-finite ones
-            // are replaced by the block's diagonal)
+            // Unconverged estimates are shifts all the same (and non-finite ones
+            // are replaced by the block's diagonal) while the iteration gets on
+            cta_aberth_real(s_m, ms, s_z, mnrm, slow ? kShiftItSlow : min(kShiftIt, 6 + m / 32));
             if (tid < ms) {
                 if (!(isfinite(s_z[tid].x) && isfinite(s_z[tid].y))) s_z[tid] = make_float2(s_m[tid + tid * MLD], 0.0f);
-                s_prev[tid] = s_z[tid];
+                s_prev[tid] = make_float2(fmaf(s_z[tid].x, isc, ctr), s_z[tid].y * isc);
             }
             __syncthreads();
             if (warp == 0) {
-                const int k = warp_pair_shifts(s_z, ms, s_mnrm, s_sh, nb0);
+                const int k = warp_pair_shifts(s_z, ms, ctr, isc, s_sh, nb0);
                 if (lane == 0) {
                     s_nb = k;
                     s_prevn = ms;
