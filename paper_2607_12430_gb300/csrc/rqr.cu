@@ -228,13 +228,17 @@ __device__ __forceinline__ void tile_update(float a[3][3], Refl l, Refl r)
 }
 // First reflector of a bulge with shifts alpha +- i r (r >= 0) or alpha +- r
 // (r < 0): from the first column of (H - s1)(H - s2) for the block starting at
-// lo.  B(i, j) is element (i, j) at B[i + j ld].
+// lo.  B(i, j) is element (i, j) at B[i + j ld].  The entries are scaled by a
+// power of two to a largest of about 1 among those squared, so that the
+// products of a block far below the matrix's scale do not underflow.
 __device__ __noinline__ Refl intro_reflector(const float *B, int ld, int lo, float alpha, float r)
 {
     const float a = B[lo + lo * ld], b = B[lo + (lo + 1) * ld], c = B[(lo + 1) + lo * ld],
                 d = B[(lo + 1) + (lo + 1) * ld], e = B[(lo + 2) + (lo + 1) * ld];
-    const float am = a - alpha, dm = d - alpha;
-    float x0 = fmaf(am, am, fmaf(b, c, r * fabsf(r))), x1 = c * (am + dm), x2 = c * e;
+    const float big = fmaxf(fabsf(a - alpha), fmaxf(fabsf(r), fabsf(c)));
+    const float sc = __uint_as_float((254u - min(max(__float_as_uint(big) >> 23, 30u), 253u)) << 23);
+    const float am = (a - alpha) * sc, dm = (d - alpha) * sc, rs = r * sc, cs = c * sc;
+    const float x0 = fmaf(am, am, fmaf(b * sc, cs, rs * fabsf(rs))), x1 = cs * (am + dm), x2 = cs * (e * sc);
     const float m = fmaxf(fabsf(x0), fmaxf(fabsf(x1), fabsf(x2)));
     Refl v{0.0f, 0.0f, 0.0f};
     if (m > 0.0f) {
@@ -1652,18 +1656,26 @@ __global__ void __launch_bounds__(32) rqr_blocks_kernel(const SchurDesc<float> *
     for (int i0 = blockIdx.x; i0 < n; i0 += gridDim.x) {
         if (bst[i0] != i0) continue;
         const int m = __popc(__ballot_sync(0xffffffffu, lane < kQrTiny && i0 + lane < n && bst[min(i0 + lane, n - 1)] == i0));
+        // scaled by a power of two to a largest entry in [1, 2): the shifts of a
+        // block far below the matrix's scale are roots of products of its entries
+        float mx = 0.0f;
         for (int e = lane; e < m * m; e += 32) {
             const int a = e % m, b = e / m;
-            M[a + b * kQrTinyLd] = cplx<float>{a <= b + 1 ? T[(i0 + a) + (int64_t)(i0 + b) * n] : 0.0f, 0.0f};
+            const float t = a <= b + 1 ? T[(i0 + a) + (int64_t)(i0 + b) * n] : 0.0f;
+            M[a + b * kQrTinyLd] = cplx<float>{t, 0.0f};
             U[a + b * kQrTinyLd] = cplx<float>{a == b ? 1.0f : 0.0f, 0.0f};
+            mx = fmaxf(mx, fabsf(t));
         }
+        const unsigned ex = min(max(__reduce_max_sync(0xffffffffu, __float_as_uint(mx)) >> 23, 1u), 253u);
+        const float sc = __uint_as_float((254u - ex) << 23), isc = __uint_as_float(ex << 23);
+        for (int e = lane; e < m * m; e += 32) M[e % m + (e / m) * kQrTinyLd].x *= sc;
         __syncwarp();
         int nsw = 0, nrot = 0;
         const bool ok = warp_tiny_schur<float, kQrTinyLd>(M, U, m, &nsw, &nrot);
         __syncwarp();
         for (int e = lane; e < m * m; e += 32) {
             const int a = e % m, b = e / m;
-            d.T[(i0 + a) + (int64_t)(i0 + b) * d.ld] = a <= b ? M[a + b * kQrTinyLd] : cplx<float>{0.0f, 0.0f};
+            d.T[(i0 + a) + (int64_t)(i0 + b) * d.ld] = a <= b ? isc * M[a + b * kQrTinyLd] : cplx<float>{0.0f, 0.0f};
             ub[(i0 + a) * kQrTiny + b] = U[a + b * kQrTinyLd];
         }
         if (lane == 0) {

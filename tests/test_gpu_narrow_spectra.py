@@ -76,3 +76,27 @@ def test_batch_of_narrow_spectra():
     for X, A in zip(Xs, As):
         X = X.cpu().numpy()
         assert oracle.rel_err(X @ X, A) <= 1e-12
+
+
+@pytest.mark.parametrize("p", [1e-10, 1e-18, 1e-22, 1e-26])
+@pytest.mark.parametrize("n", [30, 50, 130, 224, 300])
+def test_block_far_below_the_scale(n, p):
+    """Two decoupled blocks, one of them p times the other in either order: the
+    reflectors that start its sweeps and the shifts of its last rows are made
+    of products of its entries, p^2.  The small block is upper Hessenberg
+    already, so that the reduction does not square it.  Each block's factor
+    holds to the bounds of a matrix of its own."""
+    k = n // 2
+    for first in (False, True):
+        g = np.random.default_rng(8900 + n)
+        A = np.zeros((n, n))
+        big = slice(k, n) if first else slice(0, k)
+        small = slice(0, k) if first else slice(k, n)
+        m = A[small, small].shape[0]
+        A[big, big] = 3.0 * np.eye(n - m) + g.standard_normal((n - m, n - m)) / np.sqrt(n - m)
+        A[small, small] = p * np.triu(3.0 * np.eye(m) + g.standard_normal((m, m)) / np.sqrt(m), -1)
+        A = A.astype(np.float32).astype(np.float64)
+        T, Q = schur32(A)
+        for b in (big, small):
+            back, orth = factor_errors(A[b, b], T[b, b], Q[b, b])
+            assert back <= 14 * np.sqrt(n) * U32 and orth <= 8 * n * U32
