@@ -66,3 +66,14 @@ def test_staged_and_cooperative_factors(helpers):
         mp.set_tuning(saved)
     back, orth = factor_errors(A, T, Q)
     assert back <= 14 * np.sqrt(n) * U32 and orth <= 8 * n * U32
+
+
+@pytest.mark.parametrize("n", [130, 200, 224, 300, 512, 1100])
+def test_reflectors_are_orthogonal_to_one_rounding(n):
+    """tau agrees with the rounded v of each reflector, so its own rounding is
+    what is left of P^T P - I: 4.1 to 5.0 sqrt(n) u and 2.7 to 3.2 n u with the
+    kernels compiled for the CPU (5.9 to 7.7 and 3.4 to 4.3 with tau = |d| / ||x||
+    as it came)."""
+    A = synth.shifted_gaussian(n, 3.0, seed=8550 + n).astype(np.float32).astype(np.float64)
+    back, orth = factor_errors(A, *schur32(A))
+    assert back <= 5.6 * np.sqrt(n) * U32 and orth <= 3.4 * n * U32
