@@ -446,7 +446,7 @@ size_t matrix_bytes(int64_t n)
 {
     const size_t nn = (size_t)n * n, cb = sizeof(cplx<R>);
     const int64_t nt = (n + 63) / 64;
-    return 5 * Carve::round(nn * cb) + Carve::round(nn * sizeof(float)) + Carve::round(nt * nt * sizeof(double)) +
+    return 5 * Carve::round(nn * cb) + Carve::round(nn * sizeof(float)) + Carve::round(std::max<int64_t>(nt * nt, xsplit_parts_cap((int)n)) * sizeof(double)) +
            Carve::round(qr_log_capacity(n) * sizeof(RotLog<R>)) + Carve::round(qr_win_capacity(n) * sizeof(WinRec)) +
            Carve::round(qr_u_capacity(n) * cb) + Carve::round((n + 8) * cb) + Carve::round(8 * sizeof(R)) +
            Carve::round(4 * sizeof(int)) + Carve::round(32 * sizeof(int)) + Carve::round(qr_win_capacity(n) * sizeof(int)) +
@@ -674,7 +674,7 @@ int batched_general(sqrtm_handle_t h, const int *idx, int count, const double *c
         cplx<R> *W = cd.take<cplx<R>>(nn), *Rt = cd.take<cplx<R>>(nn);
         float *Rhat = cd.take<float>(nn);
         const int64_t nt = (nm + 63) / 64;
-        double *partials = cd.take<double>(nt * nt);
+        double *partials = cd.take<double>(std::max<int64_t>(nt * nt, xsplit_parts_cap((int)nm)));
         SchurDesc<R> &d = hdesc[i];
         d.log = cd.take<RotLog<R>>(qr_log_capacity(nm));
         d.win = cd.take<WinRec>(qr_win_capacity(nm));
@@ -707,7 +707,7 @@ int batched_general(sqrtm_handle_t h, const int *idx, int count, const double *c
         hrj[i] = ResJob{dA[m], lda[m], dX[m], ldx[m], Rhat, partials, &q->e, &q->active, &q->norm_a, (int)nm};
         BState *hq = (BState *)host(q);
         hq->partials = partials;
-        hq->np = resid_fp64 ? residual_f64_parts((int)nm) : xsplit_parts((int)nm);
+        hq->np = resid_fp64 ? residual_f64_parts((int)nm) : xsplit_parts((int)nm, nmax, B);
     }
     SQM_CU(cudaMemcpyAsync(h->bws.p, hdr.data(), L.hdr_bytes, cudaMemcpyHostToDevice, s));
     if (!h->body_stream) SQM_CU(cudaStreamCreateWithFlags(&h->body_stream, cudaStreamNonBlocking));

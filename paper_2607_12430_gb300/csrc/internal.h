@@ -121,16 +121,18 @@ cudaError_t launch_cgemm_batched(int opA, int opB, bool a_real, int epi, const G
                                  cudaStream_t s);
 cudaError_t launch_residual_batched(const ResJob *jobs, int batch, int nmax, cudaStream_t s);
 // the same residuals from exact split-BF16 tensor-core products (xsplit.cu)
-// where these are as accurate for a matrix of norm norm_a (FP64 ones where not),
-// xsplit_parts(n) <= residual_f64_parts(n) partial sums each
-int xsplit_parts(int n);
+// where these are as accurate for a matrix of norm norm_a (FP64 ones where not);
+// xsplit_parts: partial sums of a matrix of n rows in a batch whose largest has
+// nmax, at most xsplit_parts_cap(n)
+int xsplit_parts(int n, int nmax, int batch);
+int xsplit_parts_cap(int n);
 // The general residual takes FP64 products up to n = kXsplitMinN, xsplit.cu's
 // kernel from there and tc_split.cu's (digits in global memory, TMA) from n =
 // kGenSplitMinN on.  xsplit fills at most the 152 SMs once up to n = 1024 (128
 // tiles).
 constexpr int kXsplitMinN = 32;
 constexpr int64_t kGenSplitMinN = 1025;
-// R = (A - X Y) 2^-shift; complex: Y = X, 2 xsplit_parts(n) partial sums
+// R = (A - X Y) 2^-shift; complex: Y = X.  At most 608 partial sums.
 cudaError_t launch_xsplit_residual(const double *A, int64_t lda, const double *X, int64_t ldx, const double *Y,
                                    int64_t ldy, int n, int shift, double norm_a, float *Rhat, int ldr, double *partials,
                                    int *nparts, cudaStream_t s);

@@ -37,7 +37,10 @@
 // over its own rows and columns, so that their error stays below the FP64
 // product's, and FP64 products where not (graded or far from normal X, entries
 // that are not finite) and for n <= 32, where there is less to do than the
-// digits cost.
+// digits cost.  FP64 products are bound by an SM's FP64 units (2 multiply-adds a
+// cycle), and 128 x 64 tiles leave most SMs idle, so where they do the launch has
+// up to 4 CTAs a tile, each for its own columns; those beyond the first leave
+// after the test where the tile takes the digits.
 //
 // A complex product is two real ones with 2 n terms each, the imaginary parts of
 // a row after its real ones: Re = [Xr, -Xi] [Yr; Yi], Im = [Xr, Xi] [Yi; Yr].
@@ -78,6 +81,7 @@ struct XArgs {
     double sc;
     double norm_a;  // ||A||_F: decides between the digit and the FP64 product
     int n;
+    int slices;     // CTAs per tile
 };
 
 // the scaling exponent from the largest high word of |x|: 2^r > |x| for every
@@ -191,8 +195,42 @@ __device__ __forceinline__ bool digits_accurate(const int *ri, const int *sj, in
     return (double)(mr + mc) + 0.5 * (double)log2f(sr * sc * tiles) <= 7.0 + log2(norm_a);
 }
 
-// CPLX: complex A, X, Y and Rhat (interleaved), part blockIdx.z (0 real, 1
-// imaginary) of R; leading dimensions in elements
+// jn <= NJ columns from c0 on of one row of R by FP64 products, in the order of
+// residual_f64_kernel and zresidual_f64_kernel; their sum of squares
+template <bool CPLX, int NJ>
+__device__ __forceinline__ double fp64_columns(const XArgs &a, int row, int c0, int jn, int im)
+{
+    constexpr int ES = CPLX ? 2 : 1;
+    double acc[NJ], ss = 0.0;
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) acc[j] = 0.0;
+    const double *x = a.X + ES * row;
+    const double *y = a.Y + ES * (int64_t)c0 * a.ldy;
+#pragma unroll 2
+    for (int k = 0; k < a.n; ++k) {
+        const double xv = x[ES * (int64_t)k * a.ldx];
+        const double xi = CPLX ? (im ? 1.0 : -1.0) * x[ES * (int64_t)k * a.ldx + 1] : 0.0;
+#pragma unroll
+        for (int j = 0; j < NJ; ++j) {
+            const double *yj = y + ES * (k + (int64_t)min(j, jn - 1) * a.ldy);
+            acc[j] = fma(xv, yj[im], acc[j]);
+            if (CPLX) acc[j] = fma(xi, yj[1 - im], acc[j]);
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) {
+        if (j >= jn) continue;
+        const int64_t col = c0 + j;
+        const double r = (a.A[ES * (row + col * a.lda) + im] - acc[j]) * a.sc;
+        a.Rhat[ES * (row + col * a.ldr) + im] = (float)r;
+        ss = fma(r, r, ss);
+    }
+    return ss;
+}
+
+// CPLX: complex A, X, Y and Rhat (interleaved), part blockIdx.z / slices (0 real, 1
+// imaginary) of R; leading dimensions in elements.  CTA blockIdx.z % slices of a
+// tile.
 template <bool CPLX>
 __global__ void __launch_bounds__(XT, 1)
 xsplit_residual_kernel(XArgs a, const ResJob *__restrict__ jobs)
@@ -206,17 +244,23 @@ xsplit_residual_kernel(XArgs a, const ResJob *__restrict__ jobs)
     __shared__ double s_red[XT / 32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int m0 = blockIdx.x * XM, n0 = blockIdx.y * XN;
+    const int slices = a.slices, slice = (int)blockIdx.z % slices, zi = (int)blockIdx.z / slices;
     if (jobs) {
-        const ResJob jb = jobs[blockIdx.z];
+        const ResJob jb = jobs[zi];
         if (!*jb.active) return;
         a = XArgs{jb.A, jb.X, jb.X, jb.lda, jb.ldx, jb.ldx, jb.Rhat, jb.n, jb.partials, ldexp(1.0, -2 * *jb.e),
-                  *jb.norm_a, jb.n};
+                  *jb.norm_a, jb.n, slices};
     }
     const int n = a.n;
     if (m0 >= n || n0 >= n) return;
     constexpr int ES = CPLX ? 2 : 1;  // doubles per element
-    const int im = CPLX ? (int)blockIdx.z : 0;
-    const int part = blockIdx.x + (blockIdx.y + im * cdiv_i(n, XN)) * cdiv_i(n, XM);
+    const int im = CPLX ? zi : 0;
+    const int part = (blockIdx.x + (blockIdx.y + im * cdiv_i(n, XN)) * cdiv_i(n, XM)) * slices + slice;
+    const int cz = XN / slices;  // FP64 products: columns per CTA
+    if (slice > 0 && n0 + slice * cz >= n) {
+        if (tid == 0) a.partials[part] = 0.0;
+        return;
+    }
     unsigned char *sA = (unsigned char *)(((uintptr_t)smraw + 1023) & ~(uintptr_t)1023);
     unsigned char *sB = sA + XS * XA_BYTES;
     // the scaling exponents of the tile's rows of X and columns of Y
@@ -255,34 +299,14 @@ xsplit_residual_kernel(XArgs a, const ResJob *__restrict__ jobs)
     }
     __syncthreads();
     if (!s_go) {
-        // FP64 products, in the order of residual_f64_kernel and zresidual_f64_kernel
-        double acc[16], ss = 0.0;
-#pragma unroll
-        for (int j = 0; j < 16; ++j) acc[j] = 0.0;
-        if (row < n) {
-            const double *x = a.X + ES * row;
-            const double *y = a.Y + ES * (int64_t)(n0 + 16 * cg) * a.ldy;
-            const int jn = min(16, n - n0 - 16 * cg);
-            if (jn > 0) {
-#pragma unroll 2
-                for (int k = 0; k < n; ++k) {
-                    const double xv = x[ES * (int64_t)k * a.ldx];
-                    const double xi = CPLX ? (im ? 1.0 : -1.0) * x[ES * (int64_t)k * a.ldx + 1] : 0.0;
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        const double *yj = y + ES * (k + (int64_t)min(j, jn - 1) * a.ldy);
-                        acc[j] = fma(xv, yj[im], acc[j]);
-                        if (CPLX) acc[j] = fma(xi, yj[1 - im], acc[j]);
-                    }
-                }
-            }
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-                if (j >= jn) continue;
-                const int64_t col = n0 + 16 * cg + j;
-                const double r = (a.A[ES * (row + col * a.lda) + im] - acc[j]) * a.sc;
-                a.Rhat[ES * (row + col * a.ldr) + im] = (float)r;
-                ss = fma(r, r, ss);
+        // FP64 products: columns c0 .. c0 + jn - 1 of this thread's row
+        const int c0 = n0 + slice * cz + cg * (cz / 4), jn = min(cz / 4, n - c0);
+        double ss = 0.0;
+        if (row < n && jn > 0) {
+            switch (cz / 4) {
+            case 16: ss = fp64_columns<CPLX, 16>(a, row, c0, jn, im); break;
+            case 8: ss = fp64_columns<CPLX, 8>(a, row, c0, jn, im); break;
+            default: ss = fp64_columns<CPLX, 4>(a, row, c0, jn, im); break;
             }
         }
         ss = warp_sum(ss);
@@ -293,6 +317,10 @@ xsplit_residual_kernel(XArgs a, const ResJob *__restrict__ jobs)
             for (int w = 0; w < XT / 32; ++w) t += s_red[w];
             a.partials[part] = t;
         }
+        return;
+    }
+    if (slice > 0) {  // the tile's first CTA forms it
+        if (tid == 0) a.partials[part] = 0.0;
         return;
     }
     if (tid == 0) {
@@ -422,18 +450,36 @@ xsplit_residual_kernel(XArgs a, const ResJob *__restrict__ jobs)
 
 }  // namespace
 
-int xsplit_parts(int n) { return n <= 0 ? 0 : (int)(cdiv_i(n, XM) * cdiv_i(n, XN)); }
+// CTAs per tile, at most 4 (with 16 the ones that leave cost a residual by digits
+// 6 % at n = 384): as many as fill the SMs once; for one matrix, whose tiles
+// come first in the launch and hide them, as many as give an SM the fewest
+// columns of FP64 products in a row.  A matrix of FP64 tiles alone, us with the
+// host call (about 50), one CTA a tile / this many / residual_f64_kernel: n = 64
+// 138 / 87 / 99, 128 334 / 136 / 170, 256 594 / 209 / 307, 512 1123 / 358 / 590, 640 1391
+// / 751 / 726, 777 1672 / 1111 / 1640, 1024 2181 / 2180 / 2137.
+static int xsplit_slices(int64_t tiles, bool one)
+{
+    int best = 1;
+    for (int z = 2; z <= 4; z *= 2)
+        if (z * tiles <= (one ? 4 * 152 : 152) && cdiv_i(z * tiles, 152) * best < cdiv_i(best * tiles, 152) * z) best = z;
+    return best;
+}
+static int64_t xsplit_tiles(int n) { return n <= 0 ? 0 : cdiv_i(n, XM) * cdiv_i(n, XN); }
+
+int xsplit_parts(int n, int nmax, int batch) { return (int)xsplit_tiles(n) * xsplit_slices(xsplit_tiles(nmax) * batch, false); }
+int xsplit_parts_cap(int n) { return 4 * (int)xsplit_tiles(n); }
 
 cudaError_t launch_xsplit_residual(const double *A, int64_t lda, const double *X, int64_t ldx, const double *Y,
                                    int64_t ldy, int n, int shift, double norm_a, float *Rhat, int ldr, double *partials,
                                    int *nparts, cudaStream_t s)
 {
-    *nparts = xsplit_parts(n);
+    const int z = xsplit_slices(xsplit_tiles(n), true);
+    *nparts = (int)xsplit_tiles(n) * z;
     if (n <= 0) return cudaSuccess;
     cudaError_t err = allow_max_smem((const void *)xsplit_residual_kernel<false>);
     if (err) return err;
-    xsplit_residual_kernel<false><<<dim3((unsigned)cdiv_i(n, XM), (unsigned)cdiv_i(n, XN)), XT, X_SMEM, s>>>(
-        XArgs{A, X, Y, lda, ldx, ldy, Rhat, ldr, partials, ldexp(1.0, -shift), norm_a, n}, nullptr);
+    xsplit_residual_kernel<false><<<dim3((unsigned)cdiv_i(n, XM), (unsigned)cdiv_i(n, XN), (unsigned)z), XT, X_SMEM, s>>>(
+        XArgs{A, X, Y, lda, ldx, ldy, Rhat, ldr, partials, ldexp(1.0, -shift), norm_a, n, z}, nullptr);
     count_launch();
     return cudaGetLastError();
 }
@@ -442,12 +488,13 @@ cudaError_t launch_xsplit_zresidual(const double *A, int64_t lda, const double *
                                     double norm_a, cplx<float> *Rhat, int ldr, double *partials, int *nparts,
                                     cudaStream_t s)
 {
-    *nparts = 2 * xsplit_parts(n);
+    const int z = xsplit_slices(2 * xsplit_tiles(n), true);
+    *nparts = 2 * (int)xsplit_tiles(n) * z;
     if (n <= 0) return cudaSuccess;
     cudaError_t err = allow_max_smem((const void *)xsplit_residual_kernel<true>);
     if (err) return err;
-    xsplit_residual_kernel<true><<<dim3((unsigned)cdiv_i(n, XM), (unsigned)cdiv_i(n, XN), 2), XT, X_SMEM, s>>>(
-        XArgs{A, X, X, lda, ldx, ldx, reinterpret_cast<float *>(Rhat), ldr, partials, ldexp(1.0, -shift), norm_a, n},
+    xsplit_residual_kernel<true><<<dim3((unsigned)cdiv_i(n, XM), (unsigned)cdiv_i(n, XN), 2u * z), XT, X_SMEM, s>>>(
+        XArgs{A, X, X, lda, ldx, ldx, reinterpret_cast<float *>(Rhat), ldr, partials, ldexp(1.0, -shift), norm_a, n, z},
         nullptr);
     count_launch();
     return cudaGetLastError();
@@ -458,8 +505,10 @@ cudaError_t launch_xsplit_residual_batched(const ResJob *jobs, int batch, int nm
     if (nmax <= 0 || batch <= 0) return cudaSuccess;
     cudaError_t err = allow_max_smem((const void *)xsplit_residual_kernel<false>);
     if (err) return err;
-    xsplit_residual_kernel<false><<<dim3((unsigned)cdiv_i(nmax, XM), (unsigned)cdiv_i(nmax, XN), (unsigned)batch), XT, X_SMEM,
-                             s>>>(XArgs{}, jobs);
+    XArgs a{};
+    a.slices = xsplit_slices(xsplit_tiles(nmax) * batch, false);
+    xsplit_residual_kernel<false><<<dim3((unsigned)cdiv_i(nmax, XM), (unsigned)cdiv_i(nmax, XN), (unsigned)(batch * a.slices)),
+                                    XT, X_SMEM, s>>>(a, jobs);
     count_launch();
     return cudaGetLastError();
 }

@@ -108,3 +108,29 @@ def test_complex_and_cube_root(n):
         assert i1["status"] == 0 and i2["status"] == 0
         X1, X2 = X1.cpu().numpy(), X2.cpu().numpy()
         assert np.linalg.norm(X1 - X2) <= 1e-13 * np.linalg.norm(X2)
+
+
+@pytest.mark.parametrize("n", [33, 48, 64, 65, 128, 129, 200, 257, 385, 512, 641, 1000])
+def test_every_tile_with_fp64_products(n):
+    # X X far above A: no tile takes the digits, and the columns of a tile are
+    # shared by 4 or 2 CTAs or one's own: the same products in the same order
+    g = np.random.default_rng(n)
+    X, A = g.standard_normal((n, n)), 1e-8 * g.standard_normal((n, n))
+    Ad, Xd = dev_cm(A, torch.float64), dev_cm(X, torch.float64)
+    (Rs, rs), (Rf, rf) = mp.step_residual_split(Ad, Xd, n, e=1), mp.step_residual(Ad, Xd, n, e=1)
+    assert np.array_equal(host_cm(Rs, n), host_cm(Rf, n))
+    assert rs == pytest.approx(rf, rel=n * n * U64)
+
+
+def test_batch_with_fp64_tiles():
+    # few members, so that a tile has several CTAs; moderately graded
+    As = []
+    for n in (200, 129, 70, 33, 30):
+        d = 10.0 ** np.random.default_rng(n).uniform(-1, 1, n)
+        As.append(torch.from_numpy(d[:, None] * synth.shifted_gaussian(n, 3.0, seed=n) / d[None, :]).cuda())
+    for sel in (As, As[2:], As[4:]):
+        X1, s1 = mp.sqrtm_mixed_batched(sel, kind=mp.KIND_GENERAL, steps=3)
+        X2, s2 = mp.sqrtm_mixed_batched(sel, kind=mp.KIND_GENERAL, steps=3, precision=mp.PREC_RESID_FP64)
+        assert s1 == [0] * len(sel) and s2 == s1
+        for x, y in zip(X1, X2):
+            assert oracle.rel_err(x.cpu().numpy(), y.cpu().numpy()) <= 1e-12
