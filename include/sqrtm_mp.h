@@ -150,8 +150,9 @@ typedef struct {
  *   blks          block size of the triangular square root and Sylvester
  *                 solvers, 1..32 (used when opts->blks == 0);
  *   qr_helpers    helper CTAs of the cooperative QR chase: 0 (chase CTA
- *                 alone), 1..24, or -1 (built-in rule: max(8, min(64, n/32))
- *                 for real input, 8 or from n = 1024 16 for complex);
+ *                 alone), 1..24 (the most a table may ask for), or -1
+ *                 (built-in rule: max(8, min(64, n/32)) for real input, 8 or
+ *                 from n = 1024 16 for complex);
  *   batched       sqrtm_mixed_batched: 1 sends matrices of these sizes
  *                 through the batched general path, 0 through per-matrix
  *                 calls on worker streams;

@@ -10,8 +10,9 @@ the SPD path):
 * blks -- the block size of the triangular square root and the Sylvester
   wavefront (Algorithm 1's recursion cut-off; Sec. 5 uses 32): candidates
   8, 16, 32, on sqrtm_mixed with a fixed number of corrections;
-* qr_helpers -- the helper CTAs of the cooperative QR chase (n >= 256):
-  the built-in rule (-1), 0, 8, 16;
+* qr_helpers -- the helper CTAs of the cooperative QR chase (timed for n >=
+  256; the chase takes them from n = 225, of complex matrices from 256): the
+  built-in rule (-1), 0, 8, 16;
 * spd_precision -- FP32 or split-TF32 transforms of Algorithm 3, the faster
   one among those whose forward error against the FP64 method on the same
   GPU, after SPD_STEPS corrections (the stopping test nullified, as in the

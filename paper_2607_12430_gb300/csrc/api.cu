@@ -506,7 +506,7 @@ static int general_path(sqrtm_handle_t h, const double *dA, int64_t n, int64_t l
         }
     }
     if (!real_qr)
-        SQM_CU(launch_qr_sweeps<R>(ddesc, 1, (int)n, (int *)h->staging.p + 512, qstate, s, &ms_chase, ddesc + 1, h->side,
+        SQM_CU(launch_qr_sweeps<R>(ddesc, (int)n, (int *)h->staging.p + 512, qstate, s, &ms_chase, ddesc + 1, h->side,
                                    h->qev, qsync, tune ? tune->qr_helpers : -1));
     SQM_CU(cudaEventRecord(h->ev[1], s));
     if (root == 3) SQM_CU(launch_tricbrt<R>(T, (int)n, S, (int)n, V, (int)n, (int)n, o.blks, sc.st_solve, s));

@@ -188,25 +188,24 @@ struct HessJob {
 };
 template <class R>
 cudaError_t launch_hessenberg_cluster_batched(const HessJob<R> *jobs, int count, int nmax, cudaStream_t s);
-// d_state_all: the kQrStateInts-int state blocks of all matrices, contiguous
-// (descs[b].state == d_state_all + kQrStateInts b); h_state: pinned host
-// buffer of kQrStateInts * batch ints.  ms_chase (may be null) receives the
-// summed duration of the chase kernel's launches (CUDA events on s).
-// d_desc_alt (may be null): the same matrices with a second set of log,
-// window and U buffers; then the chase rounds alternate between the two
-// sets and each round's deferred passes run on `side` (ordered by the four
+// The complex QR iteration of one matrix.  d_state: the descriptor's state
+// block; h_state: pinned host buffer of kQrStateInts ints.  ms_chase (may be
+// null) receives the summed duration of the chase kernel's launches (CUDA
+// events on s).  d_desc_alt (may be null): the same matrix with a second set
+// of log, window and U buffers; then the chase rounds alternate between the
+// two sets and each round's deferred passes run on `side` (ordered by the four
 // events qev) while the next round's chase runs on s.  The deferred passes
 // touch only T entries outside every later active block and Z, which the
 // chase never reads.  d_sync (may be null; kQrSyncInts, the descriptors'
-// `sync`): with batch == 1 and a large enough n the chase runs as one
+// `sync`): with a large enough n the chase runs as one
 // cooperative grid of a chase CTA and helper CTAs that take the
 // out-of-window updates of the active block.  helpers: number of helper
 // CTAs (0: no cooperative grid; -1: 8, 16 from n = 1024).
 constexpr int kQrStateInts = 16;
 constexpr int kQrSyncInts = 96;  // counters of a cooperative chase (d_sync)
 template <class R>
-cudaError_t launch_qr_sweeps(const SchurDesc<R> *d_desc, int batch, int nmax, int *h_state,
-                             const int *d_state_all, cudaStream_t s, float *ms_chase = nullptr,
+cudaError_t launch_qr_sweeps(const SchurDesc<R> *d_desc, int n, int *h_state, const int *d_state, cudaStream_t s,
+                             float *ms_chase = nullptr,
                              const SchurDesc<R> *d_desc_alt = nullptr, cudaStream_t side = nullptr,
                              const cudaEvent_t *qev = nullptr, int *d_sync = nullptr, int helpers = -1);
 // The same for a REAL matrix in FP32 (rqr.cu): T and Q hold the Hessenberg

@@ -2,8 +2,8 @@
 // upper triangular Schur factor T (Algorithm 2, step 1), accumulating the
 // Givens rotations into the Schur vectors Z.
 //
-// Organisation (one CTA of 512 threads per matrix for the chase, many CTAs
-// for the rest):
+// Organisation (one CTA of 512 threads for the chase, many CTAs for the rest;
+// every launch is for one matrix):
 //
 //  * Each sweep applies nb single shifts at once: nb = min(NB, (m - 2) / 4)
 //    for an active block [lo, hi] of size m, the shifts being the eigenvalues
@@ -1139,65 +1139,56 @@ __global__ void qr_finish_kernel(const SchurDesc<R> *__restrict__ descs)
 }
 
 template <class R>
-__global__ void qr_state_init_kernel(const SchurDesc<R> *__restrict__ descs, int batch)
+__global__ void qr_state_init_kernel(const SchurDesc<R> *__restrict__ desc)
 {
-    for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < batch; b += gridDim.x * blockDim.x) {
-        int *st = descs[b].state;
-        st[0] = -2;  // fresh: start from hi = n - 1
-        for (int q = 1; q < kQrStateInts; ++q) st[q] = 0;
-        // the small-block counts that qr_tiny_kernel adds up
-        if (int *c = descs[b].counters) c[5] = c[6] = 0;
-    }
+    int *st = desc->state;
+    st[0] = -2;  // fresh: start from hi = n - 1
+    for (int q = 1; q < kQrStateInts; ++q) st[q] = 0;
+    // the small-block counts that qr_tiny_kernel adds up
+    if (int *c = desc->counters) c[5] = c[6] = 0;
 }
 
 // A matrix whose iteration did not finish within the round limit gets the
 // iteration-cap status.
 template <class R>
-__global__ void qr_mark_unfinished_kernel(const SchurDesc<R> *__restrict__ descs, int batch)
+__global__ void qr_mark_unfinished_kernel(const SchurDesc<R> *__restrict__ desc)
 {
-    for (int b = blockIdx.x * blockDim.x + threadIdx.x; b < batch; b += gridDim.x * blockDim.x)
-        if (!descs[b].state[2]) atomicExch(descs[b].status, 3);
+    if (!desc->state[2]) atomicExch(desc->status, 3);
 }
 
+// about 128 row blocks, as the passes of the last round are not overlapped
+// with a chase and should spread over many SMs
 template <class R>
-int qr_rows_per_cta(int nmax, int batch)
+int qr_rows_per_cta(int n)
 {
     constexpr int RRMAX = QrDims<R>::RR;
-    size_t per = (size_t)(std::max(nmax, 1) + 1) * sizeof(cplx<R>);
-    size_t avail = 200 * 1024 - 2 * (size_t)RRMAX * RRMAX * sizeof(cplx<R>) - (size_t)std::max(nmax, 1) * sizeof(int);
-    size_t r = avail / per;
-    // one matrix: about 128 row blocks, as the passes of the last round are
-    // not overlapped with a chase and should spread over many SMs; a batch:
-    // about 8 CTAs per SM over all matrices, since every CTA reads each
-    // window's rotation product once, whatever its number of rows
-    const size_t want = batch > 1 ? (size_t)cdiv_i((int64_t)std::max(nmax, 1) * batch, 152 * 8)
-                                  : (size_t)cdiv_i(std::max(nmax, 1), 128);
-    return (int)std::max<size_t>(1, std::min<size_t>(std::min<size_t>(32, r), want));
+    size_t per = (size_t)(std::max(n, 1) + 1) * sizeof(cplx<R>);
+    size_t avail = 200 * 1024 - 2 * (size_t)RRMAX * RRMAX * sizeof(cplx<R>) - (size_t)std::max(n, 1) * sizeof(int);
+    return (int)std::max<size_t>(1, std::min<size_t>(std::min<size_t>(32, avail / per), (size_t)cdiv_i(std::max(n, 1), 128)));
 }
 
 template <class R>
-cudaError_t launch_qr_sweeps(const SchurDesc<R> *d_desc, int batch, int nmax, int *h_state,
-                             const int *d_state_all, cudaStream_t s, float *ms_chase,
+cudaError_t launch_qr_sweeps(const SchurDesc<R> *d_desc, int n, int *h_state, const int *d_state, cudaStream_t s, float *ms_chase,
                              const SchurDesc<R> *d_desc_alt, cudaStream_t side, const cudaEvent_t *qev,
                              int *d_sync, int helpers)
 {
     constexpr int RRMAX = QrDims<R>::RR;
-    const int rpc = qr_rows_per_cta<R>(nmax, batch);
+    const int rpc = qr_rows_per_cta<R>(n);
     const size_t ubytes = 2 * (size_t)RRMAX * RRMAX * sizeof(cplx<R>);
-    const size_t mbytes = (size_t)std::max(nmax, 1) * sizeof(int);  // write-back masks
-    const size_t rows_bytes = (size_t)rpc * nmax * sizeof(cplx<R>) + ubytes + mbytes;
-    const size_t cols_bytes = (size_t)rpc * (nmax + 1) * sizeof(cplx<R>) + ubytes + mbytes;
+    const size_t mbytes = (size_t)std::max(n, 1) * sizeof(int);  // write-back masks
+    const size_t rows_bytes = (size_t)rpc * n * sizeof(cplx<R>) + ubytes + mbytes;
+    const size_t cols_bytes = (size_t)rpc * (n + 1) * sizeof(cplx<R>) + ubytes + mbytes;
     cudaError_t err;
     if ((err = allow_max_smem((const void *)qr_chase_kernel<R, false>))) return err;
     if ((err = allow_max_smem((const void *)qr_chase_kernel<R, true>))) return err;
     // cooperative chase (one chase CTA + H helper CTAs) for one large matrix
-    const bool coop = d_sync != nullptr && batch == 1 && nmax >= kQrCoopMinN && helpers != 0;
-    int H = helpers > 0 ? std::min(helpers, 24) : nmax >= 1024 ? 16 : 8;  // d_sync holds 4 + H counters
+    const bool coop = d_sync != nullptr && n >= kQrCoopMinN && helpers != 0;
+    int H = helpers > 0 ? std::min(helpers, 24) : n >= 1024 ? 16 : 8;  // d_sync holds 4 + H counters
     if ((err = allow_max_smem((const void *)qr_build_u_kernel<R>))) return err;
     if ((err = allow_max_smem((const void *)qr_apply_rows_kernel<R>))) return err;
     if ((err = allow_max_smem((const void *)qr_apply_cols_kernel<R>))) return err;
-    qr_state_init_kernel<R><<<1, 256, 0, s>>>(d_desc, batch); count_launch();
-    const int ctas = (int)cdiv_i(nmax, rpc);
+    qr_state_init_kernel<R><<<1, 1, 0, s>>>(d_desc); count_launch();
+    const int ctas = (int)cdiv_i(n, rpc);
     bool all = false;
     cudaEvent_t ev[2] = {nullptr, nullptr};
     if (ms_chase) {
@@ -1219,33 +1210,29 @@ cudaError_t launch_qr_sweeps(const SchurDesc<R> *d_desc, int batch, int nmax, in
             if ((err = cudaLaunchCooperativeKernel((const void *)qr_chase_kernel<R, true>, dim3(1 + H), dim3(kQrThreads),
                                                    args, QrDims<R>::chase_smem, s))) break;
         } else {
-            qr_chase_kernel<R, false><<<batch, kQrThreads, QrDims<R>::chase_smem, s>>>(dd, 0);
+            qr_chase_kernel<R, false><<<1, kQrThreads, QrDims<R>::chase_smem, s>>>(dd, 0);
         }
         count_launch();
         if (ms_chase && (err = cudaEventRecord(ev[1], s))) break;
-        if ((err = cudaMemcpyAsync(h_state, d_state_all, sizeof(int) * kQrStateInts * batch, cudaMemcpyDeviceToHost, s))) break;
+        if ((err = cudaMemcpyAsync(h_state, d_state, sizeof(int) * kQrStateInts, cudaMemcpyDeviceToHost, s))) break;
         if ((err = cudaStreamSynchronize(s))) break;
         if (ms_chase) {
             float ms = 0.0f;
             if ((err = cudaEventElapsedTime(&ms, ev[0], ev[1]))) break;
             *ms_chase += ms;
         }
-        int maxwin = 0;
-        all = true;
-        for (int b = 0; b < batch; ++b) {
-            all = all && h_state[kQrStateInts * b + 2];
-            maxwin = std::max(maxwin, h_state[kQrStateInts * b + 7]);
-        }
-        if (maxwin > 0) {
+        all = h_state[2] != 0;
+        const int wins = h_state[7];
+        if (wins > 0) {
             cudaStream_t ds = s;
             if (overlap) {
                 if ((err = cudaEventRecord(qev[par], s)) || (err = cudaStreamWaitEvent(side, qev[par], 0))) break;
                 ds = side;
             }
-            qr_tiny_kernel<R><<<dim3(maxwin, batch), 32, 0, ds>>>(dd); count_launch();
-            qr_build_u_kernel<R><<<dim3(maxwin, batch), 128, QrDims<R>::build_smem, ds>>>(dd); count_launch();
-            qr_apply_rows_kernel<R><<<dim3(2 * ctas, batch), 256, rows_bytes, ds>>>(dd, rpc, ctas); count_launch();
-            qr_apply_cols_kernel<R><<<dim3(ctas, batch), 256, cols_bytes, ds>>>(dd, rpc); count_launch();
+            qr_tiny_kernel<R><<<wins, 32, 0, ds>>>(dd); count_launch();
+            qr_build_u_kernel<R><<<wins, 128, QrDims<R>::build_smem, ds>>>(dd); count_launch();
+            qr_apply_rows_kernel<R><<<2 * ctas, 256, rows_bytes, ds>>>(dd, rpc, ctas); count_launch();
+            qr_apply_cols_kernel<R><<<ctas, 256, cols_bytes, ds>>>(dd, rpc); count_launch();
             if (overlap) {
                 if ((err = cudaEventRecord(qev[2 + par], side))) break;
                 used[par] = true;
@@ -1261,14 +1248,14 @@ cudaError_t launch_qr_sweeps(const SchurDesc<R> *d_desc, int batch, int nmax, in
     if (ev[0]) cudaEventDestroy(ev[0]);
     if (ev[1]) cudaEventDestroy(ev[1]);
     if (err) return err;
-    if (!all) { qr_mark_unfinished_kernel<R><<<1, 256, 0, s>>>(d_desc, batch); count_launch(); }
-    qr_finish_kernel<R><<<dim3(64, batch), 256, 0, s>>>(d_desc); count_launch();
+    if (!all) { qr_mark_unfinished_kernel<R><<<1, 1, 0, s>>>(d_desc); count_launch(); }
+    qr_finish_kernel<R><<<64, 256, 0, s>>>(d_desc); count_launch();
     return cudaGetLastError();
 }
 
-template cudaError_t launch_qr_sweeps<float>(const SchurDesc<float> *, int, int, int *, const int *, cudaStream_t, float *,
+template cudaError_t launch_qr_sweeps<float>(const SchurDesc<float> *, int, int *, const int *, cudaStream_t, float *,
                                              const SchurDesc<float> *, cudaStream_t, const cudaEvent_t *, int *, int);
-template cudaError_t launch_qr_sweeps<double>(const SchurDesc<double> *, int, int, int *, const int *, cudaStream_t, float *,
+template cudaError_t launch_qr_sweeps<double>(const SchurDesc<double> *, int, int *, const int *, cudaStream_t, float *,
                                               const SchurDesc<double> *, cudaStream_t, const cudaEvent_t *, int *, int);
 
 }  // namespace sqm

@@ -135,7 +135,7 @@ static int schur_step(sqrtm_handle_t h, cplx<R> *T, cplx<R> *Q, int64_t n)
                                       tune ? tune->qr_helpers : -1))
             return 7;
     }
-    if (!real && launch_qr_sweeps<R>(dd, 1, (int)n, hstate, qstate, h->stream)) return 7;
+    if (!real && launch_qr_sweeps<R>(dd, (int)n, hstate, qstate, h->stream)) return 7;
     int st = 0;
     if (fetch(h, &st, ss.iscal + 1, sizeof(int))) return 7;
     return st;
