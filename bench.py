@@ -138,7 +138,7 @@ def _peaks():
 # the chase kernel's source it was taken with: SHA-256 of rqr.cu up to the
 # first kernel after the chase (the deferred-pass kernels and the host code
 # follow it) plus qr_small.cuh and common.cuh, else null.
-CHASE_TRAFFIC = {"sha256": "5895323f26c34b1be0d4a63237c624c7dbd5c3a6e33c575caddfd11c6b756e79", "bytes": 1638656}
+CHASE_TRAFFIC = {"sha256": "0e750d4907d78bf6602eecfeb3730e8208777613653eb8b120cbf652f8dd9c3d", "bytes": 1555968}
 _CHASE_END = "__global__ void __launch_bounds__(kBuildThreads) rqr_build_u_kernel"
 
 

@@ -42,7 +42,8 @@
 //
 // Shifts: the eigenvalues of the trailing 2 nb x 2 nb block by the
 // Ehrlich-Aberth iteration (see qr_small.cuh for the method) on the real
-// block, started from the previous sweep's, taken in conjugate pairs.
+// block less the mean of its diagonal, started from the previous sweep's, taken
+// in conjugate pairs.
 // Deflation, exceptional shifts and the iteration cap are those of qr.cu.
 #include <algorithm>
 
@@ -1097,7 +1098,10 @@ __device__ __noinline__ void helper_cta(const SchurDesc<float> &d, float *T, int
 // the steps and an estimate of the shifts per half-warp, against a fast and a
 // general copy and an estimate per warp, ms of chase: n = 64 0.35 / 0.54, 101
 // 0.83 / 0.99, 200 2.14 / 2.85, 256 3.38 / 5.48, 512 10.1 / 12.5, 1024 31.4 /
-// 32.6, 2048 97.5 / 112.9.
+// 32.6, 2048 97.5 / 112.9.  (Since then, with shifts relative to the spread and tau
+// from the rounded v, means over 4 to 12 matrices before / after: n = 64 0.44 /
+// 0.44, 101 0.79 / 0.80, 200 2.32 / 2.38, 512 9.6 / 9.7, 1024 30.2 / 30.7, 2048 100 to
+// 103 / 100 to 106.)
 template <int MODE>
 __global__ void __launch_bounds__(kCta, 1)
 rqr_chase_kernel(const SchurDesc<float> *__restrict__ descs, int H, int nlo, int nhi)
