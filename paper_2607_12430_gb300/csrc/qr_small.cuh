@@ -14,18 +14,38 @@ static constexpr int kQrTinyLd = 33;     // leading dimension of its shared-memo
 static constexpr int kAberthIt = 24;     // iteration limit of the simultaneous shift refinement
 
 // Complex Givens G = [c s; -conj(s) c] with c real and G [x; y] = [r; 0].
+// c^2 + |s|^2 = 1 to rounding only if the phase x / |x| has modulus 1, and a
+// subnormal |x| has too few bits for that (c^2 + |s|^2 came out between 0.89 and
+// 1.04 where a shift met an eigenvalue exactly), so a small x is scaled up
+// for the phase, and both where y is small too.
 template <class R>
 __device__ __forceinline__ void givens(cplx<R> x, cplx<R> y, R &c, cplx<R> &s, cplx<R> &r)
 {
+    const R up = R(1.2676506002282294e30);  // 2^100
+    const R low = sizeof(R) == 4 ? R(1e-28) : R(1e-280);
     R ax = hypot(x.x, x.y), ay = hypot(y.x, y.y);
     if (ay == R(0)) { c = 1; s = {0, 0}; r = x; return; }
-    if (ax == R(0)) { c = 0; s = {y.x / ay, -y.y / ay}; r = {ay, 0}; return; }
-    R nrm = hypot(ax, ay);
+    const cplx<R> yu = up * y;
+    if (ax == R(0)) {
+        r = {ay, 0};
+        if (ay < low) { y = yu; ay = hypot(y.x, y.y); }
+        c = 0;
+        s = {y.x / ay, -y.y / ay};
+        return;
+    }
     cplx<R> ph{x.x / ax, x.y / ax};
+    R back = R(1);
+    if (ax < low) {
+        const cplx<R> xu = up * x;
+        const R au = hypot(xu.x, xu.y);
+        ph = cplx<R>{xu.x / au, xu.y / au};
+        if (ay < low) { ax = au; y = yu; ay = hypot(y.x, y.y); back = R(1) / up; }
+    }
+    R nrm = hypot(ax, ay);
     c = ax / nrm;
     cplx<R> cy = conj(y);
     s = cplx<R>{(ph.x * cy.x - ph.y * cy.y) / nrm, (ph.x * cy.y + ph.y * cy.x) / nrm};
-    r = cplx<R>{ph.x * nrm, ph.y * nrm};
+    r = (back * nrm) * ph;
 }
 
 // Eigenvalue of [a b; c d] closer to d, written without cancellation:

@@ -58,3 +58,14 @@ def test_plain_fp64_method(n):
         X, info = mp.sqrtm_schur_fp64(torch.from_numpy(A).cuda(), kind=mp.KIND_GENERAL)
         assert info["status"] == 0
         assert oracle.rel_err(X.cpu().numpy(), oracle.sqrtm_schur(A)) <= 1e-12
+
+
+@pytest.mark.parametrize("n,shift", [(25, 3.0), (28, 3.0), (32, 48.707), (33, 3.0), (34, 17.727), (35, 6.425), (35, 14.2),
+                                     (36, 3.0), (40, 3.0), (64, 20.0)])
+def test_rotations_of_vanishing_entries(n, shift):
+    # shift I + a cycle: where a shift meets an eigenvalue exactly, the first
+    # entry of a rotation is subnormal and its phase needs scaling
+    A = shift * np.eye(n) + np.roll(np.eye(n), 1, axis=0)
+    X, info = mp.sqrtm_mixed_complex(torch.from_numpy(A.T.astype(np.complex128).copy()).cuda())
+    assert info["status"] == 0
+    assert oracle.rel_err(X.cpu().numpy().T, oracle.sqrtm_schur(A)) <= 1e-12
