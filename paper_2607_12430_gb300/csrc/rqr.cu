@@ -69,7 +69,7 @@ constexpr int kStep = 352;           // threads that take part in a step (11 war
 constexpr int kQuad = 128;           // threads of a group that applies a window to 32 segments
 constexpr int KB = 4;                // steps between two barriers of such a group
 constexpr int NAH = 11;              // column triples ahead of the chain
-constexpr int kShiftIt = 12;         // iterations of the shift refinement (of a large active block)
+constexpr int kShiftIt = 12;         // iterations of the shift refinement
 constexpr float kShiftTol = 3e-2f;   // and its tolerance relative to the spread of the estimates
 constexpr int kShiftSlow = 6;        // after this many sweeps without deflation the refinement starts anew
 constexpr int kShiftItSlow = 30;     // and may take this many iterations
@@ -621,10 +621,11 @@ __device__ __noinline__ bool quad_window(float *vec, int stride, bool on, const 
 // entries they ran into it as well.)  On entry z holds m distinct estimates;
 // true: the last corrections were at most kShiftTol max|z|.  Shifts need not
 // be eigenvalues to rounding: the correction that passes the test is itself
-// applied, and the iteration converges cubically.  An iteration costs about ten
-// steps of a sweep, so at most 6 + (rows of the active block) / 32 of them, up
-// to kShiftIt, are taken: ms of chase with 10 / 14 at n = 64 0.452 / 0.462, 200
-// 2.28 / 2.36, 512 9.93 / 9.86, 2048 105.2 / 106.3.
+// applied, and the iteration converges cubically.  An iteration costs about eight
+// steps of a sweep; a resident matrix, whose sweeps are short, takes at most
+// 6 + (rows of the active block) / 32 of them up to kShiftIt, the others kShiftIt
+// (ms of chase, means over 80 to 100 matrices, this rule everywhere / kShiftIt
+// everywhere: n = 101 0.805 / 0.813, 256 3.57 / 3.53, 300 4.60 / 4.51, 512 9.91 / 9.73).
 //
 // A half-warp per estimate (warps 0 .. 15 take 32), lane r of it keeping the
 // sums of rows r and r + 16, as packed pairs (re, im): the packed FP32
@@ -1259,7 +1260,7 @@ rqr_chase_kernel(const SchurDesc<float> *__restrict__ descs, int H, int nlo, int
             __syncthreads();
             // Unconverged estimates are shifts all the same (and non-finite ones
             // are replaced by the block's diagonal) while the iteration gets on
-            cta_aberth_real(s_m, ms, s_z, mnrm, slow ? kShiftItSlow : min(kShiftIt, 6 + m / 32));
+            cta_aberth_real(s_m, ms, s_z, mnrm, slow ? kShiftItSlow : MODE == 2 ? min(kShiftIt, 6 + m / 32) : kShiftIt);
             if (tid < ms) {
                 if (!(isfinite(s_z[tid].x) && isfinite(s_z[tid].y))) s_z[tid] = make_float2(s_m[tid + tid * MLD], 0.0f);
                 s_prev[tid] = make_float2(fmaf(s_z[tid].x, isc, ctr), s_z[tid].y * isc);
